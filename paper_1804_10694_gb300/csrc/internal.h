@@ -76,6 +76,44 @@ struct TcArgs {
   const unsigned* readyB;
 };
 
+// Direct convolution from halo tiles in shared memory (conv_halo.cu).
+enum HaloPass : int {
+  kHaloFirst = 0,     // unscaled, folding the image's max |x| into amaxA (beta == 0)
+  kHaloRescale = 1,   // after kHaloFirst: again with the exponent, if the image needs one
+  kHaloKnown = 2      // the maximum is known (a preparing launch took it)
+};
+struct HaloArgs {
+  int H, W, K, R, S;
+  int groups;                      // input channels / 16
+  int kn, tiles;                   // output features and 16 x 8-pixel tiles of a unit
+  int hb, wb, nb, units;           // row, column and feature blocks; units in all
+  int steps, steps_per_block, chunks;   // k-steps of a unit, of an accumulation block; filter chunks
+  int bw, px;                      // halo width and pixels
+  int load_bytes, stage_bytes, chb, slot_bytes;
+  int nstage, nslot, nw, off_bar;  // ring depths and the barrier block's offset in shared memory
+  int pass;
+  int staged;                      // outputs pass through shared memory and tmO (K a multiple of 4, out 16-byte aligned)
+  float alpha, beta;
+  float* out;
+  unsigned* amaxA;
+  const unsigned* amaxB;
+  int* err;
+  unsigned* state;                 // cleared by the last CTA of the execution's last launch
+  int state_words;
+};
+// Whether the kernel covers this convolution; fills the geometry.
+bool halo_geometry(Prec prec, int64_t batch, int64_t H, int64_t W, int64_t C, int64_t K, int R, int S,
+                   HaloArgs* out);
+// Raise the kernel variant's shared-memory limit (call outside stream capture).
+cudaError_t halo_prepare(Prec prec, const HaloArgs& a);
+// tmX: FP32 image {C, W, H, N}, boxes of 16 channels x bw x (16 + R - 1);
+// tmB: the filter's planes (rows in (channel group, tap, channel) order along
+// K), boxes of 128 bytes x kn rows; tmO (when a.staged): the FP32 output
+// {K, W, H, N}, boxes of min(kn, 32) features x 8 x 4 pixels, swizzled by a
+// box row's bytes (64 or 128).
+cudaError_t halo_launch(Prec prec, const HaloArgs& a, int grid, const CUtensorMap& tmX, const CUtensorMap& tmB,
+                        const CUtensorMap& tmO, cudaStream_t s);
+
 struct TcLaunch {
   int bn;          // tile N (64 or 128; 128 or 256 for a CTA pair; 32 for a narrow convolution)
   Prec prec;       // BF16, BF16X6 or TF32
@@ -131,16 +169,19 @@ cudaError_t scale_c_launch(int64_t M, int64_t N, float beta, float* C, int64_t l
 // A: M x K (lda) -> planesA [P][M][pitch];  B: K x N (ldb) -> planesB [P][N][pitch],
 // P = prec_planes(prec).
 // transA: A is stored K x M (lda >= M); transB: B is stored N x K (ldb >= K).
+// group_taps > 0 (B alone, a filter of group_taps x C rows, C = K / group_taps
+// a multiple of 16): the planes' K order is (16-channel group, tap, channel)
+// instead of (tap, channel).
 cudaError_t pack_launch(Prec prec, const float* A, int64_t M, int64_t K, int64_t lda, const float* B,
                         int64_t N, int64_t ldb, unsigned* amaxA, unsigned* amaxB, unsigned* cntA,
                         unsigned* cntB, void* planesA, void* planesB, int64_t pitch, int sms,
-                        cudaStream_t s, bool transA = false, bool transB = false);
+                        cudaStream_t s, bool transA = false, bool transB = false, int group_taps = 0);
 // Fused-split preparation, one launch: A's block maxima only (no planes:
 // the gemm kernel splits A itself) and B packed as by pack_launch.
 cudaError_t pack_fused_launch(Prec prec, const float* A, int64_t M, int64_t K, int64_t lda,
                               const float* B, int64_t N, int64_t ldb, unsigned* amaxA,
                               unsigned* amaxB, unsigned* cntB, void* planesB, int64_t pitch, int sms,
-                              cudaStream_t s, int64_t K_b = -1, bool transB = false);
+                              cudaStream_t s, int64_t K_b = -1, bool transB = false, int group_taps = 0);
 // A row panel of A (rows rows, starting at a 128-row block) packed into the
 // planes of the whole matrix at planesA (already offset to the panel's
 // first row; plane_stride = elements from one plane to the next).

@@ -361,6 +361,21 @@ static gemm_status encode_im2col_planes(CUtensorMap* map, Prec prec, const void*
   return GEMM_OK;
 }
 
+// An FP32 NHWC tensor itself, for the halo kernel: boxes of box_c channels x
+// box_w x box_h pixels of one image, zero outside the image on loads.
+static gemm_status encode_nhwc(CUtensorMap* map, const float* X, int64_t batch, int64_t H, int64_t W, int64_t C,
+                               int box_c, int box_w, int box_h, CUtensorMapSwizzle swizzle) {
+  cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)batch};
+  cuuint64_t strides[3] = {(cuuint64_t)(C * 4), (cuuint64_t)(W * C * 4), (cuuint64_t)(H * W * C * 4)};
+  cuuint32_t box[4] = {(cuuint32_t)box_c, (cuuint32_t)box_w, (cuuint32_t)box_h, 1};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(X), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return fail(GEMM_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d) for an NHWC tensor", (int)r);
+  return GEMM_OK;
+}
+
 gemm_status validate_shape_t(bool transA, bool transB, int64_t M, int64_t N, int64_t K, int64_t lda,
                              int64_t ldb, int64_t ldc) {
   if (M < 0 || N < 0 || K < 0) return fail(GEMM_ERR_INVALID_ARG, "negative size M=%lld N=%lld K=%lld",
@@ -401,7 +416,8 @@ static gemm_status resolve_mode(gemm_mode mode, const DeviceState& d, gemm_mode*
 
 gemm_status plan_create_impl(int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb, int64_t ldc,
                              gemm_mode mode, int config_id, gemm_select sel, gemm_plan_t* out,
-                             bool transA, bool transB, int64_t conv_image_elems, unsigned opts) {
+                             bool transA, bool transB, int64_t conv_image_elems, unsigned opts,
+                             const HaloArgs* halo) {
   if (!out) return fail(GEMM_ERR_INVALID_ARG, "null plan output pointer");
   *out = nullptr;
   const bool comp = (opts & GEMM_OPT_COMPENSATED) != 0;
@@ -446,7 +462,8 @@ gemm_status plan_create_impl(int64_t M, int64_t N, int64_t K, int64_t lda, int64
     config_id = find_config(64, p->cfg.split_k, p->cfg.kb, p->cfg.group_m);
     config_get(m, config_id, &p->cfg);
   }
-  if ((opts & kOptNarrowConv) && conv_image_elems >= 0 && !p->cfg.fused && p->cfg.cluster == 1)
+  if (halo) p->cfg.block_n = halo->kn;   // the filter's boxes hold kn rows
+  else if ((opts & kOptNarrowConv) && conv_image_elems >= 0 && !p->cfg.fused && p->cfg.cluster == 1)
     p->cfg.block_n = 32;   // a packed convolution with few output features: 128 x 32 tiles
   const int cluster = p->cfg.cluster == 2 ? 2 : 1;
   if (cluster == 2 && conv_image_elems >= 0)
@@ -474,7 +491,7 @@ gemm_status plan_create_impl(int64_t M, int64_t N, int64_t K, int64_t lda, int64
   const bool fused = p->cfg.fused != 0;
   const int np = prec_planes(pr);
   const bool conv_packed = conv_image_elems >= 0 && !fused;
-  const size_t bytesA = fused ? 0
+  const size_t bytesA = fused || halo ? 0
                         : conv_packed ? (size_t)np * conv_image_elems * es
                                       : (size_t)np * M * p->pitch * es;
   const size_t bytesB = (size_t)np * N * p->pitch * es;
@@ -499,7 +516,7 @@ gemm_status plan_create_impl(int64_t M, int64_t N, int64_t K, int64_t lda, int64
                 cudaGetErrorString(e));
   }
   char* w = static_cast<char*>(p->ws);
-  p->planesA = fused ? nullptr : w + offA;
+  p->planesA = fused || halo ? nullptr : w + offA;
   p->planesB = w + offB;
   p->amaxA = reinterpret_cast<unsigned*>(w + offAmax);
   p->amaxB = p->amaxA + nblkA;
@@ -551,7 +568,16 @@ gemm_status plan_create_impl(int64_t M, int64_t N, int64_t K, int64_t lda, int64
   p->launch.fused = fused;
   p->launch.cluster = cluster;
   p->launch.comp = comp;
-  if (cluster == 2) {
+  if (halo) {
+    p->halo = true;
+    p->hargs = *halo;
+    p->hargs.amaxA = p->amaxA;
+    p->hargs.amaxB = p->amaxB;
+    p->hargs.err = dev->err_word;
+    p->hargs.state = p->amaxA;
+    p->launch.grid = std::min(halo->units, dev->sms);
+    if ((e = halo_prepare(pr, p->hargs)) != cudaSuccess) return cuda_fail(e, "halo kernel attribute");
+  } else if (cluster == 2) {
     // one cluster per SM pair that can hold one at a time
     if ((e = tc_pair_prepare(bn, pr, &p->max_pairs)) != cudaSuccess) return cuda_fail(e, "pair kernel attribute");
     p->launch.grid = 2 * (int)std::min<int64_t>(a.num_units, p->max_pairs);
@@ -561,6 +587,54 @@ gemm_status plan_create_impl(int64_t M, int64_t N, int64_t K, int64_t lda, int64
     if ((e = tc_prepare(bn, pr, fused)) != cudaSuccess) return cuda_fail(e, "kernel attribute");
   }
   *out = p.release();
+  return GEMM_OK;
+}
+
+// A convolution plan of the halo kernel: the filter packed (and, with beta
+// != 0, the image's maximum taken), then the convolution; with beta == 0 a
+// last launch repeats it scaled when the image needs an exponent.
+static gemm_status halo_execute(gemm_plan_t p, float alpha, const float* X, const float* B, float beta, float* out,
+                                cudaStream_t s, cudaEvent_t* ev) {
+  const int64_t elems = (int64_t)p->conv_batch * p->args.conv_H * p->args.conv_W * p->args.conv_C;
+  const int taps = p->args.conv_R * p->args.conv_S;
+  cudaError_t e =
+      beta == 0.0f
+          ? pack_launch(p->prec, nullptr, 0, p->K, p->K, B, p->N, p->ldb, p->amaxA, p->amaxB, p->cntA, p->cntB,
+                        nullptr, p->planesB, p->pitch, p->sms, s, false, false, taps)
+          : pack_fused_launch(p->prec, X, 1, elems, elems, B, p->N, p->ldb, p->amaxA, p->amaxB, p->cntB,
+                              p->planesB, p->pitch, p->sms, s, p->K, false, taps);
+  if (e != cudaSuccess) return cuda_fail(e, "pack launch");
+  HaloArgs h = p->hargs;
+  CUtensorMap tmX, tmO;
+  gemm_status st = encode_nhwc(&tmX, X, p->conv_batch, h.H, h.W, p->args.conv_C, 16, h.bw, 16 + h.R - 1,
+                               CU_TENSOR_MAP_SWIZZLE_NONE);
+  if (st != GEMM_OK) return st;
+  h.staged = h.K % 4 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0;
+  if (h.staged)
+    st = encode_nhwc(&tmO, out, p->conv_batch, h.H, h.W, h.K, std::min(h.kn, 32), 8, 4,
+                     h.kn == 16 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B);
+  else
+    std::memset(&tmO, 0, sizeof tmO);
+  if (st != GEMM_OK) return st;
+  h.alpha = alpha;
+  h.beta = beta;
+  h.out = out;
+  h.pass = beta == 0.0f ? kHaloFirst : kHaloKnown;
+  h.state_words = beta == 0.0f ? 0 : p->args.state_words;
+  if (ev) cudaEventRecord(ev[1], s);
+  if ((e = halo_launch(p->prec, h, p->launch.grid, tmX, p->tmB, tmO, s)) != cudaSuccess)
+    return cuda_fail(e, "convolution launch");
+  if (beta == 0.0f) {
+    h.pass = kHaloRescale;
+    h.state_words = p->args.state_words;
+    if ((e = halo_launch(p->prec, h, p->launch.grid, tmX, p->tmB, tmO, s)) != cudaSuccess)
+      return cuda_fail(e, "convolution launch");
+  }
+  if (ev) {
+    cudaEventRecord(ev[2], s);
+    cudaEventRecord(ev[3], s);
+    ++p->prof_n;
+  }
   return GEMM_OK;
 }
 
@@ -597,6 +671,7 @@ gemm_status plan_execute_impl(gemm_plan_t p, float alpha, const float* A, const 
     // one exponent for the whole image: its max, scanned as a single row
     if (reinterpret_cast<uintptr_t>(A) % 16 != 0)
       return fail(GEMM_ERR_ALIGNMENT, "the convolution's input image must be 16-byte aligned");
+    if (p->halo) return halo_execute(p, alpha, A, B, beta, C, s, ev);
     const int64_t elems = (int64_t)p->conv_batch * p->args.conv_H * p->args.conv_W * p->args.conv_C;
     if (!p->launch.fused) {
       // packed: the image split once into planes, then B packed alone
@@ -1179,15 +1254,18 @@ gemm_status gemm_conv_plan_create(int64_t batch, int64_t H, int64_t W, int64_t C
   // the default plan of a packed convolution with at most 32 output
   // features and no split-K takes the narrow tile (128 x 32, two CTAs a SM)
   const unsigned narrow = default_choice && packed_conv && K <= 32 && c.split_k == 1 ? kOptNarrowConv : 0u;
+  HaloArgs geo{};
+  const bool halo = default_choice && packed_conv && c.split_k == 1 &&
+                    halo_geometry(prec_of_mode(mode), batch, H, W, C, K, R, S, &geo);
   gemm_plan_t p = nullptr;
   gemm_status st = plan_create_impl(M, K, Kd, Kd, K, K, mode, config_id, GEMM_SELECT_DEFAULT, &p, false,
-                                    false, packed_conv ? elems : -1, narrow);
+                                    false, packed_conv ? elems : -1, narrow, halo ? &geo : nullptr);
   if (st != GEMM_OK) return st;
   // packed: channels per im2col box (32: the two planes interleaved by
   // 16-channel groups, the only layout of tf32 planes)
   const Prec pr = prec_of_mode(mode);
   const int box_c = pr == Prec::TF32 ? 32 : C % 64 == 0 ? 64 : prec_planes(pr) == 2 ? 32 : 16;
-  if (packed_conv && (st = encode_im2col_planes(&p->tmA, p->prec, p->planesA, prec_planes(p->prec), batch, H,
+  if (packed_conv && !halo && (st = encode_im2col_planes(&p->tmA, p->prec, p->planesA, prec_planes(p->prec), batch, H,
                                                 W, C, R, S, box_c)) != GEMM_OK) {
     plan_destroy_impl(p);
     return st;

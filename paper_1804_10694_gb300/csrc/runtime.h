@@ -42,6 +42,8 @@ struct gemm_plan_s {
   CUtensorMap tmA{}, tmB{};
   gb::TcArgs args{};
   gb::TcLaunch launch{};
+  bool halo = false;                // convolution from halo tiles (no image planes)
+  gb::HaloArgs hargs{};
   int max_pairs = 0;                // CTA-pair plans: clusters resident at once
   // stage timing (gemm_plan_profile): four events per recorded execution,
   // at the start of packing, before and after the main kernel, at the end
@@ -79,11 +81,13 @@ int select_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int64_t lda, 
 constexpr unsigned kOptNarrowConv = 1u << 16;
 
 // conv_image_elems >= 0: a packed convolution, whose A planes hold the
-// split image (that many elements a plane) instead of M x pitch rows
+// split image (that many elements a plane) instead of M x pitch rows; with
+// `halo` its image is split inside the kernel and has no planes
 gemm_status plan_create_impl(int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb, int64_t ldc,
                              gemm_mode mode, int config_id, gemm_select sel, gemm_plan_t* out,
                              bool transA = false, bool transB = false,
-                             int64_t conv_image_elems = -1, unsigned opts = 0);
+                             int64_t conv_image_elems = -1, unsigned opts = 0,
+                             const HaloArgs* halo = nullptr);
 gemm_status plan_execute_impl(gemm_plan_t p, float alpha, const float* A, const float* B, float beta,
                               float* C, cudaStream_t s);
 void plan_destroy_impl(gemm_plan_t p);

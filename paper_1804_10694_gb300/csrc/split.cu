@@ -193,12 +193,21 @@ constexpr int kColTileFloats = 64 * 128;
 
 __device__ __forceinline__ int col_swizzle(int k) { return ((k >> 3) & 7) << 2; }
 
-template <Prec PR, Pass PASS>
+//
+// GROUPED (a convolution's filter, K = taps x C rows in (tap, channel)
+// order): plane column k = 16 (g taps + tap) + c holds stored row
+// tap C + 16 g + c, the (channel group, tap, channel) order.
+__device__ __forceinline__ int64_t grouped_row(int64_t k, int64_t K, int taps) {
+  const int64_t i = k >> 4, g = i / taps, tap = i - g * taps;
+  return tap * (K / taps) + 16 * g + (k & 15);
+}
+
+template <Prec PR, Pass PASS, bool GROUPED>
 __device__ __forceinline__ unsigned split_cols_tile(const float* __restrict__ X, int64_t K, int64_t N,
                                                 int64_t ld, bool vec, unsigned* __restrict__ amax,
                                                 void* __restrict__ planes, int64_t plane,
                                                 int64_t pitch, int64_t n0, int64_t k0,
-                                                float* __restrict__ tile) {
+                                                float* __restrict__ tile, int taps) {
   constexpr bool TF32 = PR == Prec::TF32;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   unsigned m = 0;
@@ -210,7 +219,7 @@ __device__ __forceinline__ unsigned split_cols_tile(const float* __restrict__ X,
       const int64_t k = k0 + w + 8 * i;
       v[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       if (k >= K || n >= N) continue;
-      const float* p = X + k * ld + n;
+      const float* p = X + (GROUPED ? grouped_row(k, K, taps) : k) * ld + n;
       if (vec && n + 3 < N) {
         v[i] = *reinterpret_cast<const float4*>(p);
       } else {
@@ -399,6 +408,7 @@ struct OpShape {
 struct PackShape {
   OpShape op[2];            // A, B
   int64_t K, pitch;
+  int taps;                 // GROUPED kernels: filter taps of B's K order
 
   __device__ int ktiles(const OpShape& o) const {
     return o.kcontig ? (int)((pitch + 255) / 256) : (int)((pitch + 63) / 64);
@@ -420,20 +430,21 @@ struct PackShape {
 };
 
 // Split item l of operand o (unscaled); returns this thread's max |x|.
-template <Prec PR>
+template <Prec PR, bool GROUPED>
 __device__ __forceinline__ unsigned op_item(const PackShape& p, const OpShape& o, int l, float* tile) {
   const int kt = p.ktiles(o);
   if (o.kcontig)
     return split_rows_tile<PR, kFirst>(o.X, o.rows, p.K, o.ld, o.vec, o.amax, o.planes, o.plane, p.pitch,
                                          (int64_t)(l / kt) * 32, (int64_t)(l % kt) * 256);
-  return split_cols_tile<PR, kFirst>(o.X, p.K, o.rows, o.ld, o.vec, o.amax, o.planes, o.plane, p.pitch,
-                                       (int64_t)(l / kt) * 128, (int64_t)(l % kt) * 64, tile);
+  return split_cols_tile<PR, kFirst, GROUPED>(o.X, p.K, o.rows, o.ld, o.vec, o.amax, o.planes, o.plane,
+                                                p.pitch, (int64_t)(l / kt) * 128, (int64_t)(l % kt) * 64, tile,
+                                                p.taps);
 }
 
-template <Prec PR>
+template <Prec PR, bool GROUPED>
 __device__ __forceinline__ unsigned first_item(const PackShape& p, int i, float* tile) {
   const int na = p.items_of(p.op[0]);
-  return i < na ? op_item<PR>(p, p.op[0], i, tile) : op_item<PR>(p, p.op[1], i - na, tile);
+  return i < na ? op_item<PR, GROUPED>(p, p.op[0], i, tile) : op_item<PR, GROUPED>(p, p.op[1], i - na, tile);
 }
 
 // The CTA that completed block b (fin: its final max bits) marks it ready
@@ -449,7 +460,7 @@ __device__ __forceinline__ void mark_block_ready(unsigned* cnt, bool resplit) {
 
 // Close a run of `run` items of block `blk` (encoded as in block_of); the
 // CTA that completes an out-of-range block re-splits it with its exponent.
-template <Prec PR>
+template <Prec PR, bool GROUPED>
 __device__ __forceinline__ void finish_op_block(const PackShape& p, const OpShape& o, int64_t b, unsigned m,
                                                 unsigned run, float* tile) {
   const int kt = p.ktiles(o);
@@ -472,42 +483,42 @@ __device__ __forceinline__ void finish_op_block(const PackShape& p, const OpShap
     const bool resplit = block_exponent(fin) != 0;
     if (resplit) {
       for (int64_t k0 = 0; k0 < p.pitch; k0 += 64)
-        split_cols_tile<PR, kRescale>(o.X, p.K, o.rows, o.ld, o.vec, o.amax, o.planes, o.plane, p.pitch,
-                                        b * 128, k0, tile);
+        split_cols_tile<PR, kRescale, GROUPED>(o.X, p.K, o.rows, o.ld, o.vec, o.amax, o.planes, o.plane,
+                                                 p.pitch, b * 128, k0, tile, p.taps);
     }
     mark_block_ready(o.cnt + b, resplit);
   }
 }
 
-template <Prec PR>
+template <Prec PR, bool GROUPED>
 __device__ __forceinline__ void finish_block(const PackShape& p, int64_t blk, unsigned m, unsigned run,
                                              float* tile) {
   if (blk >= 0)
-    finish_op_block<PR>(p, p.op[0], blk, m, run, tile);
+    finish_op_block<PR, GROUPED>(p, p.op[0], blk, m, run, tile);
   else
-    finish_op_block<PR>(p, p.op[1], -1 - blk, m, run, tile);
+    finish_op_block<PR, GROUPED>(p, p.op[1], -1 - blk, m, run, tile);
 }
 
 // Items [i0, i1) of one problem, in runs of one block each.
-template <Prec PR>
+template <Prec PR, bool GROUPED = false>
 __device__ __forceinline__ void pack_range(const PackShape& p, int i0, int i1, float* tile) {
   int i = i0;
   while (i < i1) {
     const int64_t blk = p.block_of(i);
     unsigned m = 0, run = 0;
     do {
-      m = max(m, first_item<PR>(p, i, tile));
+      m = max(m, first_item<PR, GROUPED>(p, i, tile));
       ++run;
       ++i;
     } while (i < i1 && p.block_of(i) == blk);
-    finish_block<PR>(p, blk, m, run, tile);
+    finish_block<PR, GROUPED>(p, blk, m, run, tile);
   }
 }
 
 // ------------------------------------------------ single-problem kernels
 // CTA c takes the c-th contiguous share of the items.  Four CTAs a SM (at
 // most 64 registers a thread).
-template <Prec PR>
+template <Prec PR, bool GROUPED>
 __global__ void __launch_bounds__(256, 4) pack_first_kernel(const PackShape p) {
   __shared__ __align__(16) float tile[kColTileFloats];
   // launched as a programmatic dependent of the stream's previous kernel
@@ -522,13 +533,13 @@ __global__ void __launch_bounds__(256, 4) pack_first_kernel(const PackShape p) {
   const int total = p.items();
   const int per = (total + gridDim.x - 1) / gridDim.x;
   const int i0 = blockIdx.x * per;
-  pack_range<PR>(p, i0, min(total, i0 + per), tile);
+  pack_range<PR, GROUPED>(p, i0, min(total, i0 + per), tile);
 }
 
 // Fused-split preparation in one launch: A's block maxima (grid-stride),
 // then B packed as in pack_first_kernel (p holds B only; a contiguous
 // share of its items per CTA).
-template <Prec PR, int MODE>
+template <Prec PR, int MODE, bool GROUPED = false>
 __global__ void __launch_bounds__(256, 4) fused_prep_kernel(const AmaxShape a, const PackShape p) {
   __shared__ __align__(16) float tile[kColTileFloats];
   griddep_wait();   // as pack_first_kernel
@@ -537,7 +548,7 @@ __global__ void __launch_bounds__(256, 4) fused_prep_kernel(const AmaxShape a, c
   const int total = p.items();
   const int per = (total + gridDim.x - 1) / gridDim.x;
   const int i0 = blockIdx.x * per;
-  pack_range<PR>(p, i0, min(total, i0 + per), tile);
+  pack_range<PR, GROUPED>(p, i0, min(total, i0 + per), tile);
   griddep_launch_dependents();
 }
 
@@ -727,9 +738,9 @@ OpShape make_op(const float* X, int64_t rows, int64_t ld, bool kcontig, unsigned
   return o;
 }
 
-PackShape make_shape(const OpShape& a, const OpShape& b, int64_t K, int64_t pitch) {
+PackShape make_shape(const OpShape& a, const OpShape& b, int64_t K, int64_t pitch, int taps = 0) {
   PackShape p;
-  p.op[0] = a, p.op[1] = b, p.K = K, p.pitch = pitch;
+  p.op[0] = a, p.op[1] = b, p.K = K, p.pitch = pitch, p.taps = taps;
   return p;
 }
 
@@ -743,12 +754,19 @@ cudaError_t launch_first(Prec prec, const PackShape& p, int sms, cudaStream_t s)
   if (first == 0) return cudaSuccess;
   const int grid = grid_for(first, sms);
   cudaError_t e;
-  if (prec == Prec::TF32)
-    e = launch_pdl(pack_first_kernel<Prec::TF32>, grid, 256, 0, s, p);
+  if (p.taps > 0) {
+    if (prec == Prec::TF32)
+      e = launch_pdl(pack_first_kernel<Prec::TF32, true>, grid, 256, 0, s, p);
+    else if (prec == Prec::BF16)
+      e = launch_pdl(pack_first_kernel<Prec::BF16, true>, grid, 256, 0, s, p);
+    else
+      return cudaErrorInvalidValue;
+  } else if (prec == Prec::TF32)
+    e = launch_pdl(pack_first_kernel<Prec::TF32, false>, grid, 256, 0, s, p);
   else if (prec == Prec::BF16X6)
-    e = launch_pdl(pack_first_kernel<Prec::BF16X6>, grid, 256, 0, s, p);
+    e = launch_pdl(pack_first_kernel<Prec::BF16X6, false>, grid, 256, 0, s, p);
   else
-    e = launch_pdl(pack_first_kernel<Prec::BF16>, grid, 256, 0, s, p);
+    e = launch_pdl(pack_first_kernel<Prec::BF16, false>, grid, 256, 0, s, p);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -762,21 +780,21 @@ int pack_first_items(int64_t M, int64_t N, int64_t pitch) {
 cudaError_t pack_launch(Prec prec, const float* A, int64_t M, int64_t K, int64_t lda, const float* B,
                         int64_t N, int64_t ldb, unsigned* amaxA, unsigned* amaxB, unsigned* cntA,
                         unsigned* cntB, void* planesA, void* planesB, int64_t pitch, int sms,
-                        cudaStream_t s, bool transA, bool transB) {
+                        cudaStream_t s, bool transA, bool transB, int group_taps) {
   const PackShape p = make_shape(make_op(A, M, lda, !transA, amaxA, cntA, planesA, M * pitch),
-                                 make_op(B, N, ldb, transB, amaxB, cntB, planesB, N * pitch), K, pitch);
+                                 make_op(B, N, ldb, transB, amaxB, cntB, planesB, N * pitch), K, pitch, group_taps);
   return launch_first(prec, p, sms, s);
 }
 
 cudaError_t pack_fused_launch(Prec prec, const float* A, int64_t M, int64_t K, int64_t lda,
                               const float* B, int64_t N, int64_t ldb, unsigned* amaxA,
                               unsigned* amaxB, unsigned* cntB, void* planesB, int64_t pitch, int sms,
-                              cudaStream_t s, int64_t K_b, bool transB) {
+                              cudaStream_t s, int64_t K_b, bool transB, int group_taps) {
   // K_b: rows of B when they differ from A's row length (the convolution
   // scans its image as one M = 1 row of all its elements)
   const PackShape p = make_shape(make_op(nullptr, 0, 1, true, nullptr, nullptr, nullptr, 0),
                                  make_op(B, N, ldb, transB, amaxB, cntB, planesB, N * pitch),
-                                 K_b >= 0 ? K_b : K, pitch);
+                                 K_b >= 0 ? K_b : K, pitch, group_taps);
   AmaxShape a;
   a.A = A, a.M = M, a.K = K, a.lda = lda, a.amax = amaxA, a.parts = 1;
   const int64_t nblk = (M + 127) / 128;
@@ -797,7 +815,12 @@ cudaError_t pack_fused_launch(Prec prec, const float* A, int64_t M, int64_t K, i
   if (total == 0) return cudaSuccess;
   const int grid = grid_for(total, sms);
   cudaError_t e;
-  if (prec == Prec::TF32) {
+  if (group_taps > 0) {   // the convolution's image is one contiguous row
+    if (mode != kAmaxFlat) return cudaErrorInvalidValue;
+    if (prec == Prec::TF32) e = launch_pdl(fused_prep_kernel<Prec::TF32, kAmaxFlat, true>, grid, 256, 0, s, a, p);
+    else if (prec == Prec::BF16) e = launch_pdl(fused_prep_kernel<Prec::BF16, kAmaxFlat, true>, grid, 256, 0, s, a, p);
+    else return cudaErrorInvalidValue;
+  } else if (prec == Prec::TF32) {
     if (mode == kAmaxFlat) e = launch_pdl(fused_prep_kernel<Prec::TF32, kAmaxFlat>, grid, 256, 0, s, a, p);
     else if (mode == kAmaxRowsVec) e = launch_pdl(fused_prep_kernel<Prec::TF32, kAmaxRowsVec>, grid, 256, 0, s, a, p);
     else e = launch_pdl(fused_prep_kernel<Prec::TF32, kAmaxRowsScalar>, grid, 256, 0, s, a, p);

@@ -1,0 +1,100 @@
+"""The halo-tile convolution (default plans without split-K, at least nine
+taps, C a multiple of 16) at the edges of its tiles: blocks of 16 rows and 16
+or 32 columns, feature tiles of 16, 32 and 64, ragged features, filters that
+are one row or one column, several channel groups, accumulation blocks longer
+than one fold, both output paths (staged, and straight for K not a multiple
+of 4 or a misaligned output), images that need their exponent."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import conv
+import oracle
+import paper_1804_10694_gb300 as pkg
+import workloads as W
+from gpu_helpers import TOL
+
+pytestmark = pytest.mark.gpu
+
+# batch, H, W, C, K, R, S
+SHAPES = [(1, 16, 32, 16, 16, 3, 3), (2, 17, 33, 16, 20, 3, 3), (24, 15, 31, 16, 7, 5, 3), (1, 40, 9, 16, 16, 9, 1),
+          (1, 9, 70, 16, 32, 1, 9), (18, 30, 35, 16, 33, 11, 11), (6, 70, 90, 48, 64, 3, 3), (6, 80, 96, 32, 100, 3, 3),
+          (1, 1, 1, 16, 16, 3, 3), (12, 66, 64, 64, 30, 5, 5)]
+
+
+def run(x, f, out0, alpha, beta, mode, offset=0):
+    n, H, Wd, C = x.shape
+    R, S, _, K = f.shape
+    plan = pkg.ConvPlan(n, H, Wd, C, K, R, S, mode=mode)
+    es = 2 if mode == "bf16x3" else 4
+    # no planes of the image in the workspace: the halo kernel runs (TF32's
+    # slots of an 11 x 11 halo do not fit beside 64 features' filter)
+    fits = not (mode == "tf32x3" and R == 11 and K > 32)
+    assert (plan.info()["workspace_bytes"] < 2 * es * (x.size + K * R * S * C)) == fits or x.size < 9000
+    dx, df = torch.from_numpy(x).cuda(), torch.from_numpy(f).cuda()
+    buf = torch.full((out0.size + 8,), float("nan"), device="cuda")
+    do = buf[offset:offset + out0.size]
+    do.copy_(torch.from_numpy(out0.reshape(-1)))
+    plan.execute_ptrs(alpha, dx.data_ptr(), df.data_ptr(), beta, do.data_ptr())
+    torch.cuda.synchronize()
+    plan.destroy()
+    got = buf.cpu().numpy()
+    assert np.isnan(np.delete(got, np.s_[offset:offset + out0.size])).all()   # nothing outside the output
+    return got[offset:offset + out0.size].reshape(out0.shape)
+
+
+@pytest.mark.parametrize("mode", ["bf16x3", "tf32x3"])
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("beta", [0.0, 0.5])
+def test_tile_edges(mode, shape, beta):
+    n, H, Wd, C, K, R, S = shape
+    x = W.conv_image(n, H, Wd, C, 300)
+    f = W.conv_filter(C, K, 301, R=R, S=S)
+    out0 = W.conv_image(n, H, Wd, K, 302)
+    ref = conv.conv_f64(x, f, 1.5, beta, out0)
+    for offset in ((0, 1) if x.size < 100000 else (0,)):
+        got = run(x, f, out0, 1.5, beta, mode, offset)
+        assert oracle.rel_frob(got.reshape(-1, K), ref.reshape(-1, K)) <= TOL, offset
+    xi = W.conv_image(n, H, Wd, C, 303, kind="integers")
+    fi = W.conv_filter(C, K, 304, kind="integers", R=R, S=S)
+    oi = W.conv_image(n, H, Wd, K, 305, kind="integers")
+    goti = run(xi, fi, oi, 1.0, beta * 2, mode)
+    assert np.array_equal(goti, conv.conv_f64(xi, fi, 1.0, beta * 2, oi).astype(np.float32))
+    pkg.device_error()
+
+
+@pytest.mark.parametrize("mode", ["bf16x3", "tf32x3"])
+@pytest.mark.parametrize("shift", [-100, 60])
+@pytest.mark.parametrize("beta", [0.0, 0.5])
+def test_scaled_image(mode, shift, beta):
+    """The exponent is found while the image is split (beta = 0: a second
+    launch starts over) or before (beta != 0); the plan's state is clean for
+    the ordinary image that follows."""
+    n, H, Wd, C, K = 2, 33, 40, 32, 24
+    base = W.conv_image(n, H, Wd, C, 310)
+    f = W.conv_filter(C, K, 311)
+    out0 = W.scaled(W.conv_image(n, H, Wd, K, 312), shift)
+    plan = pkg.ConvPlan(n, H, Wd, C, K, 3, 3, mode=mode)
+    df = torch.from_numpy(f).cuda()
+    for x, o in ((W.scaled(base, shift), out0), (base, out0), (W.scaled(base, shift), out0)):
+        dx, do = torch.from_numpy(x).cuda(), torch.from_numpy(o.copy()).cuda()
+        plan.execute(dx, df, do, 1.0, beta)
+        torch.cuda.synchronize()
+        ref = conv.conv_f64(x, f, 1.0, beta, o)
+        assert oracle.rel_frob(do.cpu().numpy().reshape(-1, K), ref.reshape(-1, K)) <= TOL
+    plan.destroy()
+
+
+@pytest.mark.parametrize("mode", ["bf16x3", "tf32x3"])
+def test_non_finite_pixels(mode):
+    """Inf and NaN pixels reach exactly the outputs whose window holds them."""
+    x = W.conv_image(1, 20, 37, 16, 320)
+    x[0, 3, 8, 5], x[0, 17, 36, 0] = np.inf, np.nan
+    f = W.conv_filter(16, 16, 321)
+    ref = conv.conv_f64(x, f)
+    got = run(x, f, np.zeros((1, 20, 37, 16), np.float32), 1.0, 0.0, mode)
+    assert np.array_equal(np.isfinite(got), np.isfinite(ref))
+    ok = np.isfinite(ref).all(axis=-1)
+    assert oracle.rel_frob(got[ok], ref[ok]) <= TOL
