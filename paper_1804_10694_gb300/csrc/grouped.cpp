@@ -69,7 +69,7 @@ gemm_status launch_all(gemm_grouped_plan_t p, cudaStream_t s) {
         e = scale_c_launch(p->M[i], p->N[i], q.beta, q.C, p->ldc[i], s);
       else
         e = simt_gemm_launch(p->M[i], p->N[i], p->K[i], q.alpha, q.A, p->lda[i], q.B, p->ldb[i],
-                             q.beta, q.C, p->ldc[i], s);
+                             q.beta, q.C, p->ldc[i], p->sms, s);
       if (e != cudaSuccess) return cuda_fail(e, "grouped SIMT launch");
     }
     return GEMM_OK;

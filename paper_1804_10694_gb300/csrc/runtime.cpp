@@ -657,7 +657,7 @@ gemm_status plan_execute_impl(gemm_plan_t p, float alpha, const float* A, const 
   }
   if (!A || !B) return fail(GEMM_ERR_INVALID_ARG, "null A or B");
   if (p->mode == GEMM_MODE_F32_SIMT) {
-    if ((e = simt_gemm_launch(M, N, K, alpha, A, p->lda, B, p->ldb, beta, C, p->ldc, s, p->transA,
+    if ((e = simt_gemm_launch(M, N, K, alpha, A, p->lda, B, p->ldb, beta, C, p->ldc, p->sms, s, p->transA,
                               p->transB)) != cudaSuccess)
       return cuda_fail(e, "simt gemm launch");
     return GEMM_OK;
