@@ -134,7 +134,12 @@ gemm_status gemm_f32_ex(int64_t M, int64_t N, int64_t K, float alpha, const floa
  * kernel's tile loads read each layout directly (no transposed copy), so the
  * results are bit-identical to the untransposed call on the transposed
  * matrices; a fused-split configuration chosen for a transposed A runs as
- * its packed twin. */
+ * its packed twin.  (A default BF16X3 plan of a tall thin or small product
+ * runs without a packing pass when its operands are 16-byte aligned with
+ * leading dimensions that are multiples of 4: the same bits for operands in
+ * the unscaled range, [2^-48, 2^48); outside it the exponents are taken over a
+ * tile's columns of B instead of 128, which can round the update with beta
+ * differently.) */
 gemm_status gemm_f32_t(int transA, int transB, int64_t M, int64_t N, int64_t K, float alpha,
                        const float* A, int64_t lda, const float* B, int64_t ldb, float beta, float* C,
                        int64_t ldc, gemm_mode mode, gemm_select sel, gemm_stream_t stream);

@@ -76,6 +76,29 @@ struct TcArgs {
   const unsigned* readyB;
 };
 
+// Gemm without a packing pass (tc_direct.cu): both operands loaded as FP32 by
+// TMA and split in the gemm kernel, BF16X3.  transA: A stored K x M; transB: B
+// stored N x K.
+struct DirectArgs {
+  const float* A;
+  const float* B;
+  float* C;
+  int64_t lda, ldb, ldc;
+  int M, N, K;
+  int transA, transB;
+  float alpha, beta;
+  int fold;                        // 64-deep chunks of K accumulated before a fold
+  int* err;
+  int tiles_m, tiles_n;            // set by direct_launch
+};
+// Raise the shared-memory limit of tile width bn (32 or 64; call outside
+// stream capture).
+cudaError_t direct_prepare(int bn);
+// tmA, tmB: the FP32 operands as stored, 128-byte swizzled boxes of 32 values
+// of 128 (A) or bn (B) stored rows, or of 32 where the rows run along M or N.
+cudaError_t direct_launch(int bn, const CUtensorMap& tmA, const CUtensorMap& tmB, DirectArgs a, int sms,
+                          cudaStream_t s);
+
 // Direct convolution from halo tiles in shared memory (conv_halo.cu).
 enum HaloPass : int {
   kHaloFirst = 0,     // unscaled, folding the image's max |x| into amaxA (beta == 0)

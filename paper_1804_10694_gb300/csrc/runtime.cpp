@@ -242,6 +242,32 @@ int default_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int sms) {
   return pick;
 }
 
+// Tile width of the gemm without packing for a default BF16X3 plan of the
+// single-CTA configuration c without split-K, or 0: packed.  Both in
+// microseconds, back to back on GB300: without packing, a launch and its
+// latencies, then waves of tiles at 0.45 (64 wide) or 0.38 a 32-deep item and 2
+// a tile; packed, a launch, the pack at 5.5 TB/s and the gemm at 0.6 a unit of
+// default_config's estimate.  Above one wave of tiles only up to 128 columns:
+// every column tile splits A again, which the estimate of wide products does
+// not show (4096 x 4096 x 128: 65 us against 55 packed).  Measured, packed ->
+// this: 50176 x 64 x 576 75.6 -> 37.5, 18790 x 16 x 1152 52 -> 19, 12544 x 128 x
+// 1152 44.6 -> 38, 1024^3 23.3 -> 19; kept packed: 2048 x 1024 x 512 (21.8
+// against 22.6), 60000 x 256 x 576 (131 against 144), 1060^3 (29.8 against 36).
+static int direct_tile(const gemm_config& c, int64_t M, int64_t N, int64_t K, int sms) {
+  const int64_t tm = (M + 127) / 128, items = (K + 31) / 32, chunks = (K + 63) / 64;
+  // (the packed plan's estimate, as in default_config)
+  const int64_t tiles = tm * ((N + c.block_n - 1) / c.block_n);
+  const double est = (double)((tiles + sms - 1) / sms) *
+                     (kA0 + (double)chunks * (c.block_n == 64 ? kChunk64 : kChunk128) +
+                      (c.block_n == 64 ? kEpi64 : kEpi128));
+  const double packed = 4.0 + 8.0 * (double)(M + N) * (double)K / 5.5e6 + 0.6 * est;
+  const int bn = N <= 32 ? 32 : 64;
+  const int64_t t = tm * ((N + bn - 1) / bn);
+  if (t > sms && N > 128) return 0;
+  const double direct = 4.0 + (double)((t + sms - 1) / sms) * ((double)items * (bn == 64 ? 0.45 : 0.38) + 2.0);
+  return direct < packed ? bn : 0;
+}
+
 // -------------------------------------------------------------------- plans
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 static gemm_status encode_planes(CUtensorMap* map, Prec p, void* base, int64_t rows, int64_t K,
@@ -284,20 +310,20 @@ static gemm_status encode_planes(CUtensorMap* map, Prec p, void* base, int64_t r
   return GEMM_OK;
 }
 
-// FP32 A itself for the fused-split kernel: 128-byte-wide boxes (32 floats)
-// of 128 rows, 128-byte swizzle, zero fill outside the matrix.  Needs a
-// 16-byte aligned base and lda % 4 == 0.
-static gemm_status encode_rows_f32(CUtensorMap* map, const float* A, int64_t M, int64_t K, int64_t lda) {
-  cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)M, 1};
-  cuuint64_t strides[2] = {(cuuint64_t)(lda * 4), (cuuint64_t)(M * lda * 4)};
-  cuuint32_t box[3] = {32, 128, 1};
+// An FP32 operand itself, rows x cols stored row-major: boxes of box_r rows x
+// 32 columns (128 bytes), 128-byte swizzle, zero fill outside.  Needs a 16-byte
+// aligned base and ld % 4 == 0.
+static gemm_status encode_f32(CUtensorMap* map, const float* X, int64_t rows, int64_t cols, int64_t ld, int box_r) {
+  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, 1};
+  cuuint64_t strides[2] = {(cuuint64_t)(ld * 4), (cuuint64_t)(rows * ld * 4)};
+  cuuint32_t box[3] = {32, (cuuint32_t)box_r, 1};
   cuuint32_t estr[3] = {1, 1, 1};
-  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(A), dims, strides,
-                        box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(X), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS)
-    return fail(GEMM_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d) for A, M=%lld K=%lld lda=%lld", (int)r,
-                (long long)M, (long long)K, (long long)lda);
+    return fail(GEMM_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d) for an operand, %lld x %lld", (int)r,
+                (long long)rows, (long long)cols);
   return GEMM_OK;
 }
 
@@ -444,6 +470,7 @@ gemm_status plan_create_impl(int64_t M, int64_t N, int64_t K, int64_t lda, int64
     return GEMM_OK;
   }
   p->prec = prec_of_mode(m);
+  const bool default_choice = config_id < 0 && sel == GEMM_SELECT_DEFAULT;
   if (config_id < 0) {
     config_id = select_config(m, M, N, K, lda, ldb, ldc, sel, dev->sms);
     if (config_id < 0) return fail(GEMM_ERR_INVALID_ARG, "no configuration for mode");
@@ -568,6 +595,11 @@ gemm_status plan_create_impl(int64_t M, int64_t N, int64_t K, int64_t lda, int64
   p->launch.fused = fused;
   p->launch.cluster = cluster;
   p->launch.comp = comp;
+  if (default_choice && m == GEMM_MODE_BF16X3 && conv_image_elems < 0 && !comp && sk == 1 && cluster == 1 &&
+      !fused) {
+    p->direct = direct_tile(p->cfg, M, N, K, dev->sms);
+    if (p->direct && (e = direct_prepare(p->direct)) != cudaSuccess) return cuda_fail(e, "kernel attribute");
+  }
   if (halo) {
     p->halo = true;
     p->hargs = *halo;
@@ -665,6 +697,31 @@ gemm_status plan_execute_impl(gemm_plan_t p, float alpha, const float* A, const 
   const bool prof = p->prof_n < p->prof_max;
   cudaEvent_t* ev = prof ? &p->prof_events[4 * p->prof_n] : nullptr;
   if (prof) cudaEventRecord(ev[0], s);
+  auto rows16 = [](const float* X, int64_t ld) { return ld % 4 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0; };
+  if (p->direct && rows16(A, p->lda) && rows16(B, p->ldb)) {
+    DirectArgs d{};
+    d.A = A, d.B = B, d.C = C;
+    d.lda = p->lda, d.ldb = p->ldb, d.ldc = p->ldc;
+    d.M = (int)M, d.N = (int)N, d.K = (int)K;
+    d.transA = p->transA, d.transB = p->transB;
+    d.alpha = alpha, d.beta = beta;
+    d.fold = p->args.kb;
+    d.err = p->err_word;
+    const int bn = p->direct;
+    CUtensorMap tA, tB;
+    gemm_status st = p->transA ? encode_f32(&tA, A, K, M, p->lda, 32) : encode_f32(&tA, A, M, K, p->lda, 128);
+    if (st == GEMM_OK)
+      st = p->transB ? encode_f32(&tB, B, N, K, p->ldb, bn) : encode_f32(&tB, B, K, N, p->ldb, 32);
+    if (st != GEMM_OK) return st;
+    if (prof) cudaEventRecord(ev[1], s);
+    if ((e = direct_launch(bn, tA, tB, d, p->sms, s)) != cudaSuccess) return cuda_fail(e, "tensor-core gemm launch");
+    if (prof) {
+      cudaEventRecord(ev[2], s);
+      cudaEventRecord(ev[3], s);
+      ++p->prof_n;
+    }
+    return GEMM_OK;
+  }
   // (the block maxima and counters are zero: the previous execution's gemm
   // launch cleared them)
   if (p->args.conv) {
@@ -718,7 +775,7 @@ gemm_status plan_execute_impl(gemm_plan_t p, float alpha, const float* A, const 
     if (a.vecA) {
       gemm_status st = a.conv ? encode_im2col(&tmAf, A, p->conv_batch, a.conv_H, a.conv_W, a.conv_C,
                                               a.conv_R, a.conv_S, a.conv_box_c)
-                              : encode_rows_f32(&tmAf, A, M, K, p->lda);
+                              : encode_f32(&tmAf, A, M, K, p->lda, 128);
       if (st != GEMM_OK) return st;
     }
     mapA = &tmAf;

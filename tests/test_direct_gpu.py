@@ -1,0 +1,86 @@
+"""Default BF16X3 plans that run without a packing pass (tall thin and small
+products whose rows TMA can load) at the edges of their tiles: items of 32 of
+K with remainders, tiles of 128 x 32 and 128 x 64, several tiles a CTA, every
+transpose.  The same plan takes the packed path for operands that start off a
+16-byte boundary: unscaled operands give the same bits either way."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_1804_10694_gb300 as pkg
+import workloads as W
+from gpu_helpers import TOL
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(128, 64, 32), (1, 1, 1), (129, 33, 31), (300, 100, 65), (128, 128, 260), (1024, 1024, 1024),
+          (20100, 64, 144), (20000, 16, 130), (40000, 96, 70)]
+
+
+def place(x, offset):
+    """x as stored with a leading dimension that is a multiple of 4, `offset`
+    floats past an aligned address; NaN around it."""
+    r, c = x.shape
+    ld = (c + 3) // 4 * 4
+    buf = torch.full((r * ld + 8,), float("nan"), device="cuda")
+    v = buf[offset:offset + r * ld].view(r, ld)
+    v[:, :c] = torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    return v
+
+
+def call(A, B, C0, ta, tb, alpha, beta, offset):
+    M, N = C0.shape
+    K = A.shape[1]
+    a = place(A.T if ta else A, offset)
+    b = place(B.T if tb else B, offset)
+    c = torch.from_numpy(C0.copy()).cuda()
+    pkg.gemm_f32_t(ta, tb, M, N, K, alpha, a.data_ptr(), a.stride(0), b.data_ptr(), b.stride(0), beta, c.data_ptr(), N,
+                   "bf16x3", "default", torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    return c.cpu().numpy()
+
+
+@pytest.mark.parametrize("M,N,K", SHAPES)
+@pytest.mark.parametrize("ta,tb", [(0, 0), (0, 1), (1, 0), (1, 1)])
+def test_edges(M, N, K, ta, tb):
+    A, B, C0 = W.uniform(M, K, 500), W.uniform(K, N, 501), W.uniform(M, N, 502)
+    for beta in (0.0, 0.5):
+        got, packed = (call(A, B, C0, ta, tb, 1.5, beta, offset) for offset in (0, 1))
+        assert np.array_equal(got.view(np.uint32), packed.view(np.uint32)), beta
+        assert oracle.rel_frob(got, oracle.gemm_f64(M, N, K, 1.5, A, B, beta, C0)) <= TOL
+    Ai, Bi = W.integers(M, K, 503), W.integers(K, N, 504)
+    got = call(Ai, Bi, C0, ta, tb, 1.0, 0.0, 0)
+    assert np.array_equal(got, oracle.gemm_f64(M, N, K, 1.0, Ai, Bi, 0.0, None).astype(np.float32))
+    pkg.device_error()
+
+
+@pytest.mark.parametrize("ta,tb", [(0, 0), (1, 1)])
+def test_scaled_blocks(ta, tb):
+    """Tiles whose rows or columns lie outside the unscaled range are computed
+    a second time with their exponents, tiles next to them are not; each
+    128 x 32 block against the oracle."""
+    M, N, K = 20000, 30, 100
+    A, B, C0 = W.uniform(M, K, 510), W.uniform(K, N, 511), W.uniform(M, N, 512)
+    A[128:256] = W.scaled(A[128:256], -100)
+    A[640:700] = W.scaled(A[640:700], 50)
+    for scale in (0, 60):
+        Bs = W.scaled(B, scale)
+        got = call(A, Bs, C0, ta, tb, 1.0, 0.0, 0)
+        ref = oracle.gemm_f64(M, N, K, 1.0, A, Bs, 0.0, None)
+        for r in (0, 128, 256, 512, 640, 19968):
+            assert oracle.rel_frob(got[r:r + 128], ref[r:r + 128]) <= TOL, (scale, r)
+
+
+def test_non_finite_values():
+    """Inf and NaN reach exactly the rows and columns that hold them."""
+    M, N, K = 1000, 64, 96
+    A, B = W.uniform(M, K, 520), W.uniform(K, N, 521)
+    A[3, 5], A[700, 95], B[40, 33] = np.inf, np.nan, -np.inf
+    got = call(A, B, np.zeros((M, N), np.float32), 0, 0, 1.0, 0.0, 0)
+    ref = oracle.gemm_f64(M, N, K, 1.0, A, B, 0.0, None)
+    assert np.array_equal(np.isfinite(got), np.isfinite(ref))
+    ok = np.isfinite(ref)
+    assert oracle.rel_frob(got[ok][None], ref[ok][None]) <= TOL
