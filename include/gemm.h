@@ -352,7 +352,9 @@ gemm_status gemm_autotune_best(int64_t M, int64_t N, int64_t K, int64_t lda, int
  * exact six numbers (else the heuristic), MODEL = the loaded cost model's
  * argmin (runs on the GPU; else the heuristic), EXHAUSTIVE = time every
  * candidate now.  -1 for F32_SIMT or an empty problem.  DEFAULT and TABLE
- * need no device (the heuristic assumes 152 SMs without one). */
+ * need no device (the heuristic assumes 152 SMs without one).  A BF16X3
+ * DEFAULT plan that runs without a packing pass in place of a split-K
+ * configuration reports the unsplit one that its other calls run. */
 gemm_status gemm_select_config(int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb, int64_t ldc,
                                gemm_mode mode, gemm_select sel, int* config_id);
 

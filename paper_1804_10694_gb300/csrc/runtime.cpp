@@ -242,30 +242,43 @@ int default_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int sms) {
   return pick;
 }
 
-// Tile width of the gemm without packing for a default BF16X3 plan of the
-// single-CTA configuration c without split-K, or 0: packed.  Both in
-// microseconds, back to back on GB300: without packing, a launch and its
-// latencies, then waves of tiles at 0.45 (64 wide) or 0.38 a 32-deep item and 2
-// a tile; packed, a launch, the pack at 5.5 TB/s and the gemm at 0.6 a unit of
-// default_config's estimate.  Above one wave of tiles only up to 128 columns:
-// every column tile splits A again, which the estimate of wide products does
-// not show (4096 x 4096 x 128: 65 us against 55 packed).  Measured, packed ->
-// this: 50176 x 64 x 576 75.6 -> 37.5, 18790 x 16 x 1152 52 -> 19, 12544 x 128 x
-// 1152 44.6 -> 38, 1024^3 23.3 -> 19; kept packed: 2048 x 1024 x 512 (21.8
-// against 22.6), 60000 x 256 x 576 (131 against 144), 1060^3 (29.8 against 36).
+// Tile width of the gemm without packing for a default BF16X3 plan whose
+// packed configuration is c (single CTAs), or 0: packed.  Both sides in
+// microseconds, back to back on GB300: without packing a launch and its
+// latencies (1.8 or, 64 wide, 3.2), then a wave of tiles at 0.40 (0.44) a
+// 32-deep item and 2 a tile; packed a launch, the pack at 5.5 TB/s and the gemm
+// at 0.6 a unit of default_config's estimate, within 10 % of what 128^3 to
+// 1060^3 took.  Above one wave of tiles only up to 128 columns: every column
+// tile splits A again, which the estimate of wide products does not show (4096 x
+// 4096 x 128: 65 us against 55 packed).  Measured, packed -> this: 128^3 11.2 ->
+// 5.4, 512^3 13.1 -> 10.2, 768^3 16.6 -> 13.3, 1024^3 21.9 -> 18.3, 50176 x 64 x
+// 576 75.6 -> 37.5, 18790 x 16 x 1152 52 -> 19, 12544 x 128 x 1152 43 -> 37; kept
+// packed: 512 x 512 x 1024 (14.4 against 16.0), 2048 x 1024 x 512 (21.8 against
+// 22.6), 60000 x 256 x 576 (131 against 144), 700 x 900 x 1300 (21.8 against
+// 24.6), 1060^3 (28.9 against 36).
+// A split-K configuration gives way (to the unsplit tile, for operands that TMA
+// cannot load) only where M, N and K are multiples of 4, that is where every
+// tight layout can be loaded.
 static int direct_tile(const gemm_config& c, int64_t M, int64_t N, int64_t K, int sms) {
-  const int64_t tm = (M + 127) / 128, items = (K + 31) / 32, chunks = (K + 63) / 64;
+  const int64_t chunks = (K + 63) / 64, items = (K + 31) / 32, tm = (M + 127) / 128;
+  if (c.split_k > 1 && ((M | N | K) & 3) != 0) return 0;
   // (the packed plan's estimate, as in default_config)
+  const int64_t per = (chunks + c.split_k - 1) / c.split_k, splits = (chunks + per - 1) / per;
   const int64_t tiles = tm * ((N + c.block_n - 1) / c.block_n);
-  const double est = (double)((tiles + sms - 1) / sms) *
-                     (kA0 + (double)chunks * (c.block_n == 64 ? kChunk64 : kChunk128) +
-                      (c.block_n == 64 ? kEpi64 : kEpi128));
-  const double packed = 4.0 + 8.0 * (double)(M + N) * (double)K / 5.5e6 + 0.6 * est;
-  const int bn = N <= 32 ? 32 : 64;
-  const int64_t t = tm * ((N + bn - 1) / bn);
-  if (t > sms && N > 128) return 0;
-  const double direct = 4.0 + (double)((t + sms - 1) / sms) * ((double)items * (bn == 64 ? 0.45 : 0.38) + 2.0);
-  return direct < packed ? bn : 0;
+  double est = (double)((tiles * splits + sms - 1) / sms) *
+               (kA0 + (double)per * (c.block_n == 64 ? kChunk64 : kChunk128) + (c.block_n == 64 ? kEpi64 : kEpi128));
+  if (splits > 1) est += kFix0 + kFix1 * (double)M * (double)N * (double)splits * 1e-6;
+  double best = 4.0 + 8.0 * (double)(M + N) * (double)K / 5.5e6 + 0.6 * est;
+  if (splits > 1) best *= 0.85;   // (the estimate of split 128-wide tiles is up to a fifth high)
+  int pick = 0;
+  for (int bn : {32, 64}) {
+    const int64_t t = tm * ((N + bn - 1) / bn);
+    if (t > sms && N > 128) continue;
+    const double direct =
+        (bn == 32 ? 1.8 : 3.2) + (double)((t + sms - 1) / sms) * ((double)items * (bn == 32 ? 0.40 : 0.44) + 2.0);
+    if (direct < best) best = direct, pick = bn;
+  }
+  return pick;
 }
 
 // -------------------------------------------------------------------- plans
@@ -477,6 +490,14 @@ gemm_status plan_create_impl(int64_t M, int64_t N, int64_t K, int64_t lda, int64
   }
   if (!config_get(m, config_id, &p->cfg))
     return fail(GEMM_ERR_INVALID_ARG, "configuration id %d out of range for mode %d", config_id, (int)m);
+  if (default_choice && m == GEMM_MODE_BF16X3 && conv_image_elems < 0 && !comp && p->cfg.cluster == 1) {
+    p->direct = direct_tile(p->cfg, M, N, K, dev->sms);
+    if (p->direct && p->cfg.split_k > 1) {
+      config_id = find_config(64, 1, p->cfg.kb, p->cfg.group_m);   // the same sums, unsplit
+      config_get(m, config_id, &p->cfg);
+      p->unsplit = true;
+    }
+  }
   if (transA && p->cfg.fused) {
     // the fused kernel stages rows of A: a transposed A runs as the packed twin
     config_id = find_config(p->cfg.block_n, p->cfg.split_k, p->cfg.kb, p->cfg.group_m);
@@ -595,11 +616,7 @@ gemm_status plan_create_impl(int64_t M, int64_t N, int64_t K, int64_t lda, int64
   p->launch.fused = fused;
   p->launch.cluster = cluster;
   p->launch.comp = comp;
-  if (default_choice && m == GEMM_MODE_BF16X3 && conv_image_elems < 0 && !comp && sk == 1 && cluster == 1 &&
-      !fused) {
-    p->direct = direct_tile(p->cfg, M, N, K, dev->sms);
-    if (p->direct && (e = direct_prepare(p->direct)) != cudaSuccess) return cuda_fail(e, "kernel attribute");
-  }
+  if (p->direct && (e = direct_prepare(p->direct)) != cudaSuccess) return cuda_fail(e, "kernel attribute");
   if (halo) {
     p->halo = true;
     p->hargs = *halo;
@@ -1131,7 +1148,7 @@ gemm_status host_gemm_impl(int64_t M, int64_t N, int64_t K, float alpha, const f
     cudaStream_t s;
     ~NoteUse() { note_use(p, s); }
   } note{p, s};
-  if (need_ab && p->mode != GEMM_MODE_F32_SIMT && p->args.split_k == 1 && !p->launch.fused &&
+  if (need_ab && p->mode != GEMM_MODE_F32_SIMT && p->args.split_k == 1 && !p->unsplit && !p->launch.fused &&
       host_panels() > 1 &&
       M >= 4 * 128 && page_locked(A) && page_locked(C))
     return host_gemm_panels(p, alpha, A, B, beta, C, s);

@@ -43,6 +43,7 @@ struct gemm_plan_s {
   gb::TcArgs args{};
   gb::TcLaunch launch{};
   int direct = 0;                   // tile width of the gemm without packing for aligned operands, or 0
+  bool unsplit = false;             // ... in place of a split-K configuration
   bool halo = false;                // convolution from halo tiles (no image planes)
   gb::HaloArgs hargs{};
   int max_pairs = 0;                // CTA-pair plans: clusters resident at once

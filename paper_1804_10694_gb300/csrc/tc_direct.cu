@@ -55,7 +55,7 @@ constexpr int kEpiWarp0 = 16, kMmaWarp = 20, kLoadWarp = 21;
 constexpr int kRegsSplit = 80, kRegsEpi = 120, kRegsCtrl = 40;
 static_assert(kGroups * kRegsSplit + kRegsEpi + kRegsCtrl <= 6 * 80, "register split");
 constexpr int kKI = 32;                    // K of an item
-constexpr int kStages = 4, kDirSlots = 4;
+constexpr int kStages = kGroups, kDirSlots = kGroups;   // a group's items all pass through the same of each
 constexpr int kVerdicts = 16;
 // bytes between 16-byte chunks of an item, 32 modulo 128: the stores of eight
 // lanes (four chunks of two stored rows) fall into different banks
@@ -66,7 +66,7 @@ template <int BN>
 struct DirCfg {
   static constexpr int CHB_BK = BN * 16 + 32;                 // K-major B
   static constexpr int A_PLANE = 8704;                        // 16 chunks of kChbMn, 4 of kChbK
-  static constexpr int B_PLANE = BN == 64 ? 4352 : 2304;
+  static constexpr int B_PLANE = (BN / 8 * kChbMn + 127) / 128 * 128;
   static constexpr int SLOT = 2 * (A_PLANE + B_PLANE);
   static constexpr int ITEM_A = 128 * kKI * 4, ITEM = (128 + BN) * kKI * 4;   // FP32 bytes
   static constexpr int EPI_PITCH = 33;

@@ -16,7 +16,7 @@ from gpu_helpers import TOL
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = [(128, 64, 32), (1, 1, 1), (129, 33, 31), (300, 100, 65), (128, 128, 260), (1024, 1024, 1024),
+SHAPES = [(128, 64, 32), (512, 512, 512), (640, 260, 300), (1, 1, 1), (129, 33, 31), (300, 100, 65), (128, 128, 260), (1024, 1024, 1024),
           (20100, 64, 144), (20000, 16, 130), (40000, 96, 70)]
 
 
