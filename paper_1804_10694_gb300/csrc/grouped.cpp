@@ -135,6 +135,28 @@ void destroy_graph(gemm_grouped_plan_t p) {
   p->graph = nullptr;
 }
 
+// Order in which the persistent CTAs take the units: long and short ones mixed so
+// that the running mean of their k-chunks stays at the mean of all.  A long unit
+// leaves the epilogue warps idle and a short one the loads and the tensor cores;
+// the accumulator ring lets the short ones' updates of C run under the long ones'
+// products.  The shortest units, one a CTA, come last and even out the end.
+std::vector<GroupedUnit> interleave_units(const std::vector<GroupedUnit>& by_k, int sms) {
+  const size_t n = by_k.size(), last = std::min(n, static_cast<size_t>(sms));
+  std::vector<GroupedUnit> out;
+  out.reserve(n);
+  size_t lo = 0, hi = n - last;   // by_k[lo, hi): longest first, still to be placed
+  int64_t total = 0, sum = 0;
+  for (size_t i = 0; i < hi; ++i) total += by_k[i].chunks;
+  const int64_t count = hi;
+  for (int64_t placed = 0; lo < hi; ++placed) {
+    const GroupedUnit& u = sum * count <= total * placed ? by_k[lo++] : by_k[--hi];
+    sum += u.chunks;
+    out.push_back(u);
+  }
+  out.insert(out.end(), by_k.end() - last, by_k.end());
+  return out;
+}
+
 }  // namespace
 
 // Grouped configuration for a set of shapes under a selection policy.
@@ -308,6 +330,7 @@ gemm_status grouped_create_impl(int G, const int64_t* M, const int64_t* N, const
       units.push_back(GroupedUnit{slot, first_m + r % rows, r / rows, g.chunks});
     }
   }
+  units = interleave_units(units, p->sms);
   if (!units.empty() &&
       (e = cudaMemcpy(p->d_units, units.data(), units.size() * sizeof(GroupedUnit), cudaMemcpyHostToDevice)) != cudaSuccess)
     return cuda_fail(e, "upload of the unit table");
