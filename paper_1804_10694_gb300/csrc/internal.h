@@ -89,13 +89,20 @@ struct DirectArgs {
   float alpha, beta;
   int fold;                        // 64-deep chunks of K accumulated before a fold
   int* err;
-  int tiles_m, tiles_n;            // set by direct_launch
+  int tiles_m, tiles_n, turned;    // set by direct_launch (its DirectGrid)
 };
-// Raise the shared-memory limit of tile width bn (32 or 64; call outside
-// stream capture).
-cudaError_t direct_prepare(int bn);
+// Tiles of a product: tiles_m x tiles_n of 128 rows x bn columns, and `turned`
+// ones of 64 rows x 128 columns for the rows below them.
+struct DirectGrid {
+  int64_t tiles_m, tiles_n, turned;
+  int64_t units() const { return tiles_m * tiles_n + turned; }
+};
+DirectGrid direct_grid(int bn, int64_t M, int64_t N, int sms);
+// Raise the shared-memory limit of tile width bn (32 or 64, with turned tiles or
+// without; call outside stream capture).
+cudaError_t direct_prepare(int bn, bool turned);
 // tmA, tmB: the FP32 operands as stored, 128-byte swizzled boxes of 32 values
-// of 128 (A) or bn (B) stored rows, or of 32 where the rows run along M or N.
+// of 128 (A; bn in a launch with turned tiles) or bn (B) stored rows, or of 32 where the rows run along M or N.
 cudaError_t direct_launch(int bn, const CUtensorMap& tmA, const CUtensorMap& tmB, DirectArgs a, int sms,
                           cudaStream_t s);
 

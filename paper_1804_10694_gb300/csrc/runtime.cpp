@@ -255,7 +255,8 @@ int default_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int sms) {
 // 576 75.6 -> 37.5, 18790 x 16 x 1152 52 -> 19, 12544 x 128 x 1152 43 -> 37; kept
 // packed: 512 x 512 x 1024 (14.4 against 16.0), 2048 x 1024 x 512 (21.8 against
 // 22.6), 60000 x 256 x 576 (131 against 144), 700 x 900 x 1300 (21.8 against
-// 24.6), 1060^3 (28.9 against 36).
+// 24.6).  1060^3 took 29.3 packed, 36 in two waves of tiles here and 22.9 in one,
+// its last rows in turned tiles (direct_grid); 1088^3 26.6 -> 21.3.
 // A split-K configuration gives way (to the unsplit tile, for operands that TMA
 // cannot load) only where M, N and K are multiples of 4, that is where every
 // tight layout can be loaded.
@@ -272,7 +273,7 @@ static int direct_tile(const gemm_config& c, int64_t M, int64_t N, int64_t K, in
   if (splits > 1) best *= 0.85;   // (the estimate of split 128-wide tiles is up to a fifth high)
   int pick = 0;
   for (int bn : {32, 64}) {
-    const int64_t t = tm * ((N + bn - 1) / bn);
+    const int64_t t = direct_grid(bn, M, N, sms).units();
     if (t > sms && N > 128) continue;
     const double direct =
         (bn == 32 ? 1.8 : 3.2) + (double)((t + sms - 1) / sms) * ((double)items * (bn == 32 ? 0.40 : 0.44) + 2.0);
@@ -616,7 +617,10 @@ gemm_status plan_create_impl(int64_t M, int64_t N, int64_t K, int64_t lda, int64
   p->launch.fused = fused;
   p->launch.cluster = cluster;
   p->launch.comp = comp;
-  if (p->direct && (e = direct_prepare(p->direct)) != cudaSuccess) return cuda_fail(e, "kernel attribute");
+  if (p->direct) {
+    const bool turned = direct_grid(p->direct, M, N, p->sms).turned != 0;
+    if ((e = direct_prepare(p->direct, turned)) != cudaSuccess) return cuda_fail(e, "kernel attribute");
+  }
   if (halo) {
     p->halo = true;
     p->hargs = *halo;
@@ -725,8 +729,9 @@ gemm_status plan_execute_impl(gemm_plan_t p, float alpha, const float* A, const 
     d.fold = p->args.kb;
     d.err = p->err_word;
     const int bn = p->direct;
+    const bool turned = direct_grid(bn, M, N, p->sms).turned != 0;
     CUtensorMap tA, tB;
-    gemm_status st = p->transA ? encode_f32(&tA, A, K, M, p->lda, 32) : encode_f32(&tA, A, M, K, p->lda, 128);
+    gemm_status st = p->transA ? encode_f32(&tA, A, K, M, p->lda, 32) : encode_f32(&tA, A, M, K, p->lda, turned ? bn : 128);
     if (st == GEMM_OK)
       st = p->transB ? encode_f32(&tB, B, N, K, p->ldb, bn) : encode_f32(&tB, B, K, N, p->ldb, 32);
     if (st != GEMM_OK) return st;

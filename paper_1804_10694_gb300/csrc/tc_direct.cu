@@ -16,6 +16,10 @@
 //     plan takes this kernel for the calls whose rows TMA can load and the packed
 //     path for the others.
 //
+// Turned tiles: the last rows of A, at most 64, may be computed transposed (see
+// direct_grid): the operands change places, the products keep their order, and the
+// sums leave along the rows of C.
+//
 // Scaling: a tile covers all of K, so its split warps see the maximum of its
 // 128 rows of A and BN columns of B; if either lies outside the unscaled range
 // the tile is computed once more with the exponents (nothing has been stored
@@ -90,24 +94,22 @@ __device__ __forceinline__ uint64_t desc_plain(uint32_t saddr, uint32_t lbo, uin
 // (K-major: the operand's rows; MN-major: piece by piece of 32 rows, its k), in
 // the 128-byte swizzle.  A split thread's unit n is the quarter row t + 128 n:
 // eight values, read as two 16-byte accesses free of bank conflicts, which
-// become a 16-byte chunk of each plane at dst[n].
-template <int N>
+// become a 16-byte chunk of each plane.
 struct Units {
-  uint32_t src0, dst[N];   // the first half's place; unit n is 4096 n bytes on
+  uint32_t src0;         // the first half's place; unit n is 4096 n bytes on
+  uint32_t dst0, step;   // unit n's chunk: dst0 + n * step
 };
-template <int N>
-__device__ __forceinline__ Units<N> make_units(bool mn, uint32_t chb, int t) {
-  Units<N> u;
+__device__ __forceinline__ Units make_units(bool mn, uint32_t chb_k, int t) {
+  Units u;
   const int r = t / 4, j = t % 4;
   u.src0 = r * 128 + ((2 * j) ^ (r & 7)) * 16;
-#pragma unroll
-  for (int n = 0; n < N; ++n)
-    u.dst[n] = mn ? (4 * n + j) * chb + r * 16 : j * chb + (r + 32 * n) * 16;
+  u.dst0 = j * (mn ? kChbMn : chb_k) + r * 16;
+  u.step = mn ? 4 * kChbMn : 32 * 16;
   return u;
 }
 
 template <int N>
-__device__ __forceinline__ void read_units(float (&v)[N][8], const uint8_t* src, const Units<N>& u) {
+__device__ __forceinline__ void read_units(float (&v)[N][8], const uint8_t* src, const Units& u) {
 #pragma unroll
   for (int n = 0; n < N; ++n) {
     const float4 a = *reinterpret_cast<const float4*>(src + (u.src0 + 4096 * n));
@@ -144,7 +146,7 @@ __device__ __forceinline__ float max_units(const float (&v)[N][8]) {
 // Splits the units' values (times sf; m: their maximum) into hi parts at dst and
 // lo parts `plane` bytes further on.
 template <int N>
-__device__ __forceinline__ void write_units(float (&v)[N][8], float m, const Units<N>& u, uint8_t* dst, uint32_t plane,
+__device__ __forceinline__ void write_units(float (&v)[N][8], float m, const Units& u, uint8_t* dst, uint32_t plane,
                                             float sf) {
   if (sf != 1.0f) {
 #pragma unroll
@@ -157,17 +159,45 @@ __device__ __forceinline__ void write_units(float (&v)[N][8], float m, const Uni
   for (int n = 0; n < N; ++n) {
     uint4 h, l;
     split_chunk_bf16(v[n], finite, h, l);
-    *reinterpret_cast<uint4*>(dst + u.dst[n]) = h;
-    *reinterpret_cast<uint4*>(dst + u.dst[n] + plane) = l;
+    *reinterpret_cast<uint4*>(dst + (u.dst0 + n * u.step)) = h;
+    *reinterpret_cast<uint4*>(dst + (u.dst0 + n * u.step) + plane) = l;
   }
 }
 
+// Epilogue of a turned tile: this thread's sums are those of column col of C, in
+// rows row0 .. row0 + BN - 1; a warp's accesses are 128 contiguous bytes of a row.
 template <int BN>
+__device__ __forceinline__ void store_turned(float (&S)[BN], const DirectArgs& a, int e, int row0, int col) {
+  const int rows = col < a.N ? a.M - row0 : 0;
+  float alpha = a.alpha;
+  if (e != 0) {   // (as epilogue_store)
+#pragma unroll
+    for (int i = 0; i < BN; ++i) S[i] = scale_pow2(alpha * S[i], e);
+    alpha = 1.0f;
+  }
+  const float* in = a.C + static_cast<int64_t>(row0) * a.ldc + col;
+  float* out = const_cast<float*>(in);
+#pragma unroll
+  for (int j = 0; j < BN; j += 8) {
+    float old[8];
+    if (a.beta != 0.0f) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k, in += a.ldc) old[k] = j + k < rows ? *in : 0.0f;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k, out += a.ldc)
+      if (j + k < rows) *out = a.beta != 0.0f ? fmaf(alpha, S[j + k], a.beta * old[k]) : alpha * S[j + k];
+  }
+}
+
+// TURN: launches with turned tiles.
+template <int BN, bool TURN>
 __global__ void __launch_bounds__(kDirThreads, 1)
     tc_direct_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const DirectArgs a) {
   using Cfg = DirCfg<BN>;
   constexpr int NACC = Cfg::NACC;
+  constexpr int BOX_A = TURN ? BN : 128;   // rows of a K-major box of the operand in A's place
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t sbase = (raw + 1023u) & ~1023u;
@@ -217,13 +247,24 @@ __global__ void __launch_bounds__(kDirThreads, 1)
   griddep_launch_dependents();
 
   const int items = (a.K + kKI - 1) / kKI;
-  const int units = a.tiles_m * a.tiles_n;
+  const int plain = a.tiles_m * a.tiles_n;
+  const int units = plain + (TURN ? a.turned : 0);
   const int fold = a.fold * (64 / kKI);
-  // tile of unit u: rows fastest, so that CTAs running together share columns of B
+  // tile of unit u: rows fastest, so that CTAs running together share columns of B.
+  // Returns whether it is turned: 128 columns of B from m0 on take A's place and
+  // the last rows of A, from n0 on, take B's (the product transposed).
   auto tile = [&](int u, int& m0, int& n0) {
+    if (TURN && u >= plain) {
+      m0 = (u - plain) * 128, n0 = a.tiles_m * 128;
+      return true;
+    }
     const int tn = u / a.tiles_m;
     m0 = (u - tn * a.tiles_m) * 128, n0 = tn * BN;
+    return false;
   };
+  // whether the operand in A's (B's) place runs along M or N in its rows
+  auto mn_a = [&](bool turned) { return turned ? a.transB == 0 : a.transA != 0; };
+  auto mn_b = [&](bool turned) { return turned ? a.transA != 0 : a.transB == 0; };
   // a unit's exponents, once its maxima are known (seq: the CTA's unit count)
   auto exponents = [&](int seq, int& eA, int& eB) {
     const volatile unsigned* v = vmax + 2 * (seq % kVerdicts);
@@ -239,25 +280,30 @@ __global__ void __launch_bounds__(kDirThreads, 1)
       bool ok = true;
       for (int u = blockIdx.x; ok && u < units; u += gridDim.x) {
         int m0, n0;
-        tile(u, m0, n0);
+        const bool turned = tile(u, m0, n0);
+        const bool mnA = mn_a(turned), mnB = mn_b(turned);
+        const CUtensorMap* const mapA = turned ? &tmB : &tmA;
+        const CUtensorMap* const mapB = turned ? &tmA : &tmB;
         for (int c = 0; c < items; ++c, ++it) {
           const uint32_t s = it % kStages;
           if (!(ok = mbar_wait(sempty(s), ((it / kStages) & 1u) ^ 1u, abort_flag, err))) break;
           const uint32_t dst = sbase + s * Cfg::ITEM;
           mbar_arrive_expect_tx(sfull(s), Cfg::ITEM);
           // boxes of 32 stored values: the operand's rows, or pieces of 32 rows of k
-          if (a.transA) {
+          if (mnA) {
 #pragma unroll
-            for (int b = 0; b < 4; ++b) tma_load_3d(dst + b * 4096, &tmA, sfull(s), m0 + 32 * b, kKI * c, 0);
+            for (int b = 0; b < 4; ++b) tma_load_3d(dst + b * 4096, mapA, sfull(s), m0 + 32 * b, kKI * c, 0);
           } else {
-            tma_load_3d(dst, &tmA, sfull(s), kKI * c, m0, 0);
+#pragma unroll
+            for (int b = 0; b < 128; b += BOX_A)
+              tma_load_3d(dst + b * 128, mapA, sfull(s), kKI * c, m0 + b, 0);
           }
-          if (a.transB) {
-            tma_load_3d(dst + Cfg::ITEM_A, &tmB, sfull(s), kKI * c, n0, 0);
+          if (!mnB) {
+            tma_load_3d(dst + Cfg::ITEM_A, mapB, sfull(s), kKI * c, n0, 0);
           } else {
 #pragma unroll
             for (int b = 0; b < BN / 32; ++b)
-              tma_load_3d(dst + Cfg::ITEM_A + b * 4096, &tmB, sfull(s), n0 + 32 * b, kKI * c, 0);
+              tma_load_3d(dst + Cfg::ITEM_A + b * 4096, mapB, sfull(s), n0 + 32 * b, kKI * c, 0);
           }
         }
       }
@@ -270,18 +316,27 @@ __global__ void __launch_bounds__(kDirThreads, 1)
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------ MMA issuer
     if (elect_one()) {
-      const uint32_t idesc = idesc_f32acc(false, 128, BN) | (a.transA ? 1u << 15 : 0u) |
-                             (a.transB ? 0u : 1u << 16);   // MN-major operands
       const uint32_t s0 = sbase + Cfg::OFF_SLOT;
-      const uint64_t dA0 = a.transA ? desc_plain(s0, 128, kChbMn) : desc_plain(s0, kChbK, 128);
-      const uint64_t dB0 = a.transB ? desc_plain(s0 + 2 * Cfg::A_PLANE, Cfg::CHB_BK, 128)
-                                    : desc_plain(s0 + 2 * Cfg::A_PLANE, 128, kChbMn);
-      const uint32_t stepA = (a.transA ? 256 : 2 * kChbK) >> 4, stepB = (a.transB ? 2 * Cfg::CHB_BK : 256) >> 4;
       constexpr uint32_t loA = Cfg::A_PLANE >> 4, loB = Cfg::B_PLANE >> 4;
+      uint32_t idesc, stepA, stepB, a1, b1, a2, b2;
+      uint64_t dA0, dB0;
+      auto set_roles = [&](bool turned) {
+        const bool mnA = mn_a(turned), mnB = mn_b(turned);
+        idesc = idesc_f32acc(false, 128, BN) | (mnA ? 1u << 15 : 0u) | (mnB ? 1u << 16 : 0u);
+        dA0 = mnA ? desc_plain(s0, 128, kChbMn) : desc_plain(s0, kChbK, 128);
+        dB0 = mnB ? desc_plain(s0 + 2 * Cfg::A_PLANE, 128, kChbMn)
+                  : desc_plain(s0 + 2 * Cfg::A_PLANE, Cfg::CHB_BK, 128);
+        stepA = (mnA ? 256 : 2 * kChbK) >> 4, stepB = (mnB ? 256 : 2 * Cfg::CHB_BK) >> 4;
+        // the packed kernel's products in its order: lo*hi, hi*lo, hi*hi (of A and B)
+        a1 = turned ? 0 : loA, b1 = turned ? loB : 0, a2 = turned ? loA : 0, b2 = turned ? 0 : loB;
+      };
+      set_roles(false);
       uint32_t it = 0, ab = 0, aph = 0;
       int seq = 0;
       bool ok = true, any = false;
       for (int u = blockIdx.x; ok && u < units; u += gridDim.x, ++seq) {
+        const bool turned = TURN && u >= plain;
+        if (TURN) set_roles(turned);
         for (int pass = 0; ok && pass < 2; ++pass) {
           for (int c0 = 0; ok && c0 < items; c0 += fold) {
             const int c1 = min(c0 + fold, items);
@@ -292,11 +347,10 @@ __global__ void __launch_bounds__(kDirThreads, 1)
               if (!(ok = mbar_wait(full(s), (it / kDirSlots) & 1u, abort_flag, err))) break;
               tc_fence_after();
               uint64_t da = dA0 + s * (Cfg::SLOT >> 4), db = dB0 + s * (Cfg::SLOT >> 4);
-              // the packed kernel's products in its order: lo*hi, hi*lo, hi*hi
 #pragma unroll
               for (int kk = 0; kk < kKI / 16; ++kk) {
-                umma_bf16(d, da + loA, db, idesc, c > c0 || kk > 0 ? 1u : 0u);
-                umma_bf16(d, da, db + loB, idesc, 1u);
+                umma_bf16(d, da + a1, db + b1, idesc, c > c0 || kk > 0 ? 1u : 0u);
+                umma_bf16(d, da + a2, db + b2, idesc, 1u);
                 umma_bf16(d, da, db, idesc, 1u);
                 da += stepA, db += stepB;
               }
@@ -331,8 +385,8 @@ __global__ void __launch_bounds__(kDirThreads, 1)
     bool ok = true;
     for (int u = blockIdx.x; ok && u < units; u += gridDim.x, ++seq) {
       int m0, n0;
-      tile(u, m0, n0);
-      {
+      const bool turned = tile(u, m0, n0);
+      if (!turned) {
         const int row = m0 + q * 32 + lane;
         if (a.beta != 0.0f && row < a.M) {
           const float* rp = a.C + static_cast<int64_t>(row) * a.ldc + n0;
@@ -382,6 +436,10 @@ __global__ void __launch_bounds__(kDirThreads, 1)
         if ((eA | eB) == 0) break;
       }
       if (!ok) break;
+      if (turned) {
+        store_turned<BN>(S, a, e, n0, m0 + q * 32 + lane);
+        continue;
+      }
       EpiView v;
       v.M = a.M, v.N = a.N, v.C = a.C, v.ldc = a.ldc, v.alpha = a.alpha, v.beta = a.beta;
       v.amaxA = v.amaxB = nullptr, v.partial = nullptr, v.split_k = 1, v.amaxA_stride = 0;
@@ -392,14 +450,14 @@ __global__ void __launch_bounds__(kDirThreads, 1)
     constexpr int NA = 4, NB = BN / 32;                // eight-value units of a thread
     const int t = threadIdx.x % kSplitThreads;
     const uint32_t g = warp >> 2;                      // group: items g, g + 4, ... of the CTA's run
-    const Units<NA> ua = make_units<NA>(a.transA != 0, a.transA ? kChbMn : kChbK, t);
-    const Units<NB> ub = make_units<NB>(a.transB == 0, a.transB ? Cfg::CHB_BK : kChbMn, t);
+    Units ua = make_units(mn_a(false), kChbK, t), ub = make_units(mn_b(false), Cfg::CHB_BK, t);
     uint32_t it = 0, st = 0;                           // items written to slots, items staged
     int seq = 0;
     bool ok = true;
     for (int u = blockIdx.x; ok && u < units; u += gridDim.x, ++seq) {
       int m0, n0;
-      tile(u, m0, n0);
+      const bool turned = tile(u, m0, n0);
+      if (TURN) ua = make_units(mn_a(turned), kChbK, t), ub = make_units(mn_b(turned), Cfg::CHB_BK, t);
       float sfA = 1.0f, sfB = 1.0f;
       float mA = 0.0f, mB = 0.0f;
       for (int pass = 0; ok && pass < 2; ++pass) {
@@ -415,8 +473,11 @@ __global__ void __launch_bounds__(kDirThreads, 1)
             read_units<NA>(va, smem + sg * Cfg::ITEM, ua);
             read_units<NB>(vb, smem + sg * Cfg::ITEM + Cfg::ITEM_A, ub);
           } else {
-            fetch_units<NA>(va, a.A, a.lda, a.M, a.K, a.transA != 0, m0, kKI * c, t);
-            fetch_units<NB>(vb, a.B, a.ldb, a.N, a.K, a.transB == 0, n0, kKI * c, t);
+            int tt = turned;   // (opaque: selected here, not held in registers through the loop)
+            asm volatile("" : "+r"(tt));
+            const bool tu = tt != 0;
+            fetch_units<NA>(va, tu ? a.B : a.A, tu ? a.ldb : a.lda, tu ? a.N : a.M, a.K, mn_a(tu), m0, kKI * c, t);
+            fetch_units<NB>(vb, tu ? a.A : a.B, tu ? a.lda : a.ldb, tu ? a.M : a.N, a.K, mn_b(tu), n0, kKI * c, t);
           }
           const float uA = max_units<NA>(va), uB = max_units<NB>(vb);
           mA = fmaxf(mA, uA), mB = fmaxf(mB, uB);
@@ -479,7 +540,7 @@ __global__ void __launch_bounds__(kDirThreads, 1)
   }
 }
 
-template <int BN>
+template <int BN, bool TURN>
 cudaError_t direct_variant(bool launch, const CUtensorMap* tmA, const CUtensorMap* tmB, const DirectArgs& a, int grid,
                            cudaStream_t s) {
   using Cfg = DirCfg<BN>;
@@ -488,7 +549,7 @@ cudaError_t direct_variant(bool launch, const CUtensorMap* tmA, const CUtensorMa
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (configured_device != dev) {
-    e = cudaFuncSetAttribute(tc_direct_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
+    e = cudaFuncSetAttribute(tc_direct_kernel<BN, TURN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
     if (e != cudaSuccess) return e;
     configured_device = dev;
   }
@@ -503,27 +564,47 @@ cudaError_t direct_variant(bool launch, const CUtensorMap* tmA, const CUtensorMa
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, tc_direct_kernel<BN>, *tmA, *tmB, a);
+  e = cudaLaunchKernelEx(&cfg, tc_direct_kernel<BN, TURN>, *tmA, *tmB, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t direct_dispatch(bool launch, int bn, const CUtensorMap* tmA, const CUtensorMap* tmB, const DirectArgs& a,
                             int grid, cudaStream_t s) {
-  if (bn == 32) return direct_variant<32>(launch, tmA, tmB, a, grid, s);
-  if (bn == 64) return direct_variant<64>(launch, tmA, tmB, a, grid, s);
+  if (bn == 32) return direct_variant<32, false>(launch, tmA, tmB, a, grid, s);
+  if (bn == 64 && a.turned) return direct_variant<64, true>(launch, tmA, tmB, a, grid, s);
+  if (bn == 64) return direct_variant<64, false>(launch, tmA, tmB, a, grid, s);
   return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
-cudaError_t direct_prepare(int bn) { return direct_dispatch(false, bn, nullptr, nullptr, DirectArgs{}, 0, nullptr); }
+cudaError_t direct_prepare(int bn, bool turned) {
+  DirectArgs a{};
+  a.turned = turned;
+  return direct_dispatch(false, bn, nullptr, nullptr, a, 0, nullptr);
+}
+
+// A turned tile covers 64 rows x 128 columns where a plain one covers 128 x 64, so
+// where at most 64 rows are left after the whole row tiles, turned ones need half
+// as many tiles for them.  They are used where that saves a wave: 1060^3 has 9 x 17
+// = 153 plain tiles on 152 SMs, or 8 x 17 + 9 = 145.
+DirectGrid direct_grid(int bn, int64_t M, int64_t N, int sms) {
+  DirectGrid g{(M + 127) / 128, (N + bn - 1) / bn, 0};
+  const int64_t rest = M % 128;
+  if (bn == 64 && rest > 0 && rest <= 64) {
+    const DirectGrid t{M / 128, g.tiles_n, (N + 127) / 128};
+    if ((t.units() + sms - 1) / sms < (g.units() + sms - 1) / sms) return t;
+  }
+  return g;
+}
 
 cudaError_t direct_launch(int bn, const CUtensorMap& tmA, const CUtensorMap& tmB, DirectArgs a, int sms,
                           cudaStream_t s) {
-  a.tiles_m = (a.M + 127) / 128;
-  a.tiles_n = (a.N + bn - 1) / bn;
-  const int64_t units = static_cast<int64_t>(a.tiles_m) * a.tiles_n;
-  return direct_dispatch(true, bn, &tmA, &tmB, a, static_cast<int>(std::min<int64_t>(units, sms)), s);
+  const DirectGrid g = direct_grid(bn, a.M, a.N, sms);
+  a.tiles_m = static_cast<int>(g.tiles_m);
+  a.tiles_n = static_cast<int>(g.tiles_n);
+  a.turned = static_cast<int>(g.turned);
+  return direct_dispatch(true, bn, &tmA, &tmB, a, static_cast<int>(std::min<int64_t>(g.units(), sms)), s);
 }
 
 }  // namespace gb

@@ -84,3 +84,24 @@ def test_non_finite_values():
     assert np.array_equal(np.isfinite(got), np.isfinite(ref))
     ok = np.isfinite(ref)
     assert oracle.rel_frob(got[ok][None], ref[ok][None]) <= TOL
+
+
+@pytest.mark.parametrize("ta,tb", [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize("M,N,K", [(1060, 1060, 100), (1088, 1028, 1060), (1025, 1080, 36), (820, 1470, 260)])
+def test_turned_tiles(M, N, K, ta, tb):
+    """More 128 x 64 tiles than SMs, but not with the last rows (up to 64) in
+    tiles of 64 x 128 whose operands change places: the packed path's bits."""
+    A, B, C0 = W.uniform(M, K, 520), W.uniform(K, N, 521), W.uniform(M, N, 522)
+    for beta in (0.0, 0.5):
+        got, packed = (call(A, B, C0, ta, tb, 1.5, beta, offset) for offset in (0, 1))
+        assert np.array_equal(got.view(np.uint32), packed.view(np.uint32)), beta
+        assert oracle.rel_frob(got, oracle.gemm_f64(M, N, K, 1.5, A, B, beta, C0)) <= TOL
+    # scaled rows in the last strip and scaled columns: the second pass of both kinds of tile
+    last = M // 128 * 128
+    A[last:] = W.scaled(A[last:], -100)
+    B[:, 130:200] = W.scaled(B[:, 130:200], 60)
+    got, want = call(A, B, C0, ta, tb, 1.5, 0.0, 0), oracle.gemm_f64(M, N, K, 1.5, A, B, 0.0, None)
+    for r in (slice(0, last), slice(last, M)):
+        for c in (slice(0, 130), slice(130, 200), slice(200, N)):
+            assert oracle.rel_frob(got[r, c], want[r, c]) <= TOL, (r, c)
+    pkg.device_error()
