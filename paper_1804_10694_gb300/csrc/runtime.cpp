@@ -206,7 +206,7 @@ constexpr double kFix0 = 4.0, kFix1 = 0.99;                           // split-K
 constexpr double kSix = 1.6;                                          // six products a chunk
 }  // namespace
 
-int default_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int sms) {
+int default_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int sms, int max_split) {
   if (config_count(mode) == 0) return -1;
   const Prec p = prec_of_mode(mode);
   const bool six = mode == GEMM_MODE_BF16X6;
@@ -226,7 +226,7 @@ int default_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int sms) {
     const int64_t slots = std::max(1, sms / t.cluster);
     const double chunk = t.chunk * (six ? kSix : 1.0);
     for (int sk : splits) {
-      if (sk > 1 && sk > chunks) break;
+      if (sk > 1 && (sk > chunks || sk > max_split)) break;
       const int64_t per = (chunks + sk - 1) / sk;
       const int64_t splits_eff = (chunks + per - 1) / per;   // (no empty split)
       const int64_t waves = (tiles * splits_eff + slots - 1) / slots;
@@ -836,10 +836,12 @@ struct CacheKey {
   int dev;
   int64_t M, N, K, lda, ldb, ldc;
   int mode, sel, trans;
+  int config;               // configuration id, or -1: by sel
   uintptr_t stream;
   bool operator<(const CacheKey& o) const {
-    return std::tie(dev, M, N, K, lda, ldb, ldc, mode, sel, trans, stream) <
-           std::tie(o.dev, o.M, o.N, o.K, o.lda, o.ldb, o.ldc, o.mode, o.sel, o.trans, o.stream);
+    return std::tie(dev, M, N, K, lda, ldb, ldc, mode, sel, trans, config, stream) <
+           std::tie(o.dev, o.M, o.N, o.K, o.lda, o.ldb, o.ldc, o.mode, o.sel, o.trans, o.config,
+                    o.stream);
   }
   bool operator==(const CacheKey& o) const { return !(*this < o) && !(o < *this); }
 };
@@ -880,11 +882,11 @@ static bool stream_capturing(cudaStream_t s) {
 
 gemm_status cached_plan(int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb, int64_t ldc,
                         gemm_mode mode, gemm_select sel, cudaStream_t s, gemm_plan_t* out,
-                        bool transA, bool transB) {
+                        bool transA, bool transB, int config = -1) {
   int dev = 0;
   cudaGetDevice(&dev);
   CacheKey key{dev, M, N, K, lda, ldb, ldc, (int)mode, (int)sel, (transA ? 1 : 0) | (transB ? 2 : 0),
-               reinterpret_cast<uintptr_t>(s)};
+               config, reinterpret_cast<uintptr_t>(s)};
   // (the capture status is read first: while this thread's stream is being
   // captured, no event of an eager execution is queried)
   const bool capturing = stream_capturing(s);
@@ -905,7 +907,7 @@ gemm_status cached_plan(int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ld
                 "no cached plan for this shape and stream while the stream is being captured: "
                 "call once before the capture, or capture an explicit plan (gemm_plan_create)");
   gemm_plan_t p = nullptr;
-  gemm_status st = plan_create_impl(M, N, K, lda, ldb, ldc, mode, -1, sel, &p, transA, transB);
+  gemm_status st = plan_create_impl(M, N, K, lda, ldb, ldc, mode, config, sel, &p, transA, transB);
   if (st != GEMM_OK) return st;
   cudaError_t e = cudaEventCreateWithFlags(&p->last_use, cudaEventDisableTiming);
   if (e != cudaSuccess) {
@@ -1047,6 +1049,38 @@ static gemm_status host_streams(int nevents) {
   return GEMM_OK;
 }
 
+// 128-row tiles of a panel; an even number if the plan's tiles are 256 rows.
+static int64_t panel_tiles(int64_t tiles_m, int64_t npan, int64_t cl) {
+  return ((tiles_m + npan - 1) / npan + cl - 1) / cl * cl;
+}
+
+// Configuration of a plan that the pipelined path runs panel by panel: the best
+// one for a panel, where the one for the whole product has its tiles (-1).  A
+// panel of 256 rows of 4096^3 is 16 pair tiles of the whole product's
+// configuration, on 16 of 76 SM pairs: 80 us behind copies of 45 us.  In 128 x 64
+// tiles it takes the whole chip, and the copies are what the call waits for:
+// 4096^3 with beta != 0 1643 -> 1291 us (same bits).  A product whose own configuration splits
+// K or splits A in the kernel keeps the unpipelined path.
+static gemm_status host_panel_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb, int64_t ldc,
+                                     int* config) {
+  *config = -1;
+  DeviceState* dev;
+  int devidx;
+  gemm_mode m;
+  gemm_status st = device_state(&dev, &devidx);
+  if (st == GEMM_OK) st = resolve_mode(mode, *dev, &m);
+  if (st != GEMM_OK) return st;
+  gemm_config whole, panel;
+  const int w = m == GEMM_MODE_F32_SIMT ? -1 : select_config(m, M, N, K, lda, ldb, ldc, GEMM_SELECT_DEFAULT, dev->sms);
+  if (w < 0 || !config_get(m, w, &whole) || whole.split_k > 1 || whole.fused) return GEMM_OK;
+  const int64_t tiles_m = (M + 127) / 128;
+  const int64_t rows = 128 * panel_tiles(tiles_m, std::min<int64_t>(host_panels(), tiles_m), whole.cluster == 2 ? 2 : 1);
+  const int c = default_config(m, rows, N, K, dev->sms, 1);
+  if (c >= 0 && config_get(m, c, &panel) && (panel.block_n != whole.block_n || panel.cluster != whole.cluster))
+    *config = c;
+  return GEMM_OK;
+}
+
 // Pipelined path: tensor-core plan without split-K, M spanning >= 2 panels.
 static gemm_status host_gemm_panels(gemm_plan_t p, float alpha, const float* A, const float* B,
                                     float beta, float* C, cudaStream_t s) {
@@ -1055,7 +1089,7 @@ static gemm_status host_gemm_panels(gemm_plan_t p, float alpha, const float* A, 
   const int npan = (int)std::min<int64_t>(host_panels(), tiles_m);
   // 128-row tiles per panel; even for a CTA-pair plan (its tiles are 256 rows)
   const int64_t cl = p->launch.cluster == 2 ? 2 : 1;
-  const int64_t tiles_per = ((tiles_m + npan - 1) / npan + cl - 1) / cl * cl;
+  const int64_t tiles_per = panel_tiles(tiles_m, npan, cl);
   gemm_status st = host_streams(2 + 2 * npan);
   if (st != GEMM_OK) return st;
   cudaEvent_t* ev = t_host.ev.data();
@@ -1143,7 +1177,10 @@ gemm_status host_gemm_impl(int64_t M, int64_t N, int64_t K, float alpha, const f
   if ((st = grow(&t_host.B, &t_host.nB, std::max<size_t>(nB, 1))) != GEMM_OK) return st;
   if ((st = grow(&t_host.C, &t_host.nC, nC)) != GEMM_OK) return st;
   gemm_plan_t p = nullptr;
-  if ((st = cached_plan(M, N, K, lda, ldb, ldc, mode, GEMM_SELECT_DEFAULT, s, &p, false, false)) != GEMM_OK)
+  const bool panels = need_ab && host_panels() > 1 && M >= 4 * 128 && page_locked(A) && page_locked(C);
+  int config = -1;
+  if (panels && (st = host_panel_config(mode, M, N, K, lda, ldb, ldc, &config)) != GEMM_OK) return st;
+  if ((st = cached_plan(M, N, K, lda, ldb, ldc, mode, GEMM_SELECT_DEFAULT, s, &p, false, false, config)) != GEMM_OK)
     return st;
   const CachedPlanUse hold(p);
   // (every path below synchronises its streams before returning, so the plan
@@ -1153,9 +1190,7 @@ gemm_status host_gemm_impl(int64_t M, int64_t N, int64_t K, float alpha, const f
     cudaStream_t s;
     ~NoteUse() { note_use(p, s); }
   } note{p, s};
-  if (need_ab && p->mode != GEMM_MODE_F32_SIMT && p->args.split_k == 1 && !p->unsplit && !p->launch.fused &&
-      host_panels() > 1 &&
-      M >= 4 * 128 && page_locked(A) && page_locked(C))
+  if (panels && p->mode != GEMM_MODE_F32_SIMT && p->args.split_k == 1 && !p->unsplit && !p->launch.fused)
     return host_gemm_panels(p, alpha, A, B, beta, C, s);
   cudaError_t e;
   if (need_ab) {
