@@ -5,11 +5,11 @@
 //
 // Host side of the plan: the problem table (tensor maps, plane addresses,
 // sizes) is written to device memory once; problems are ordered by
-// decreasing K so that the persistent CTAs, which walk the global tile list
-// in a fixed stride, take the longest tiles first and the short ones fill the
-// tail.  Per-execution values (A, B, C pointers, alpha, beta) live in a
-// second small table that is re-uploaded only when it changes, ahead of the
-// graph launch on the same stream.
+// decreasing K, and the persistent CTAs, which take the units of the tile list
+// in turn, meet the longest tiles first and the short ones fill the tail
+// (long lists are interleaved: interleave_units).  Per-execution values (A, B,
+// C pointers, alpha, beta) live in a second small table that is re-uploaded only
+// when it changes, ahead of the graph launch on the same stream.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -139,9 +139,14 @@ void destroy_graph(gemm_grouped_plan_t p) {
 // that the running mean of their k-chunks stays at the mean of all.  A long unit
 // leaves the epilogue warps idle and a short one the loads and the tensor cores;
 // the accumulator ring lets the short ones' updates of C run under the long ones'
-// products.  The shortest units, one a CTA, come last and even out the end.
+// products.  The shortest units, one a CTA, come last and even out the end.  512
+// problems of 32..1024 (3568 units): 322 -> 308 us a call, 300 of them 220 -> 210,
+// 512 of 32..512 158 -> 152.  Below eight units a CTA the order is the even-out
+// itself, and longest first stays: 712 units 117.5 against 119.8 us interleaved
+// (TF32x3), 275 units 42.1 against 42.8.
 std::vector<GroupedUnit> interleave_units(const std::vector<GroupedUnit>& by_k, int sms) {
-  const size_t n = by_k.size(), last = std::min(n, static_cast<size_t>(sms));
+  const size_t n = by_k.size(), last = static_cast<size_t>(sms);
+  if (n < 8 * last) return by_k;
   std::vector<GroupedUnit> out;
   out.reserve(n);
   size_t lo = 0, hi = n - last;   // by_k[lo, hi): longest first, still to be placed

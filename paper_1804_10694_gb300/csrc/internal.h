@@ -261,7 +261,7 @@ struct GroupedUnit {
 struct GroupedArgs {
   const GroupedProblem* probs;
   const GroupedPtrs* ptrs;
-  const GroupedUnit* units;   // num_units entries, problems longest-K first
+  const GroupedUnit* units;   // num_units entries, in the order they are taken
   int G, num_units, kb, group_m;
   int* err;
   int* unit_ctr;              // units taken so far (zero before the launch)
