@@ -26,30 +26,47 @@ def _select(s) -> int:
     return SELECTS[s] if isinstance(s, str) else int(s)
 
 
+_torch = None
+
+
+def _import_torch():
+    """torch, imported by the first call that needs it."""
+    global _torch
+    import torch
+    _torch = torch
+    return torch
+
+
 def _stream_handle(stream) -> int | None:
+    # the current stream's handle without a Stream object around it (3.1 us of a
+    # call of 13: a 512^3 product takes 10 on the GPU)
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream or None
+        c = (_torch or _import_torch())._C
+        return c._cuda_getCurrentRawStream(c._cuda_getDevice()) or None
     if isinstance(stream, int):
         return stream or None
     return stream.cuda_stream or None
 
 
 def _matrix(t, name: str):
-    import torch
+    torch = _torch or _import_torch()
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
-    if t.dtype != torch.float32:
+    if t.dtype is not torch.float32:
         raise TypeError(f"{name} must be float32")
     if not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
-    if t.dim() != 2:
+    shape = t.shape
+    if len(shape) != 2:
         raise ValueError(f"{name} must be 2-D")
-    rows, cols = t.shape
-    if rows > 0 and cols > 0 and t.stride(1) != 1:
+    rows, cols = shape
+    s0, s1 = t.stride()
+    if s1 != 1 and rows > 0 and cols > 0:
         raise ValueError(f"{name} must have unit inner stride (row-major)")
-    ld = t.stride(0) if rows > 1 else max(cols, 1)
-    return t.data_ptr(), rows, cols, max(ld, cols, 1)
+    ld = s0 if rows > 1 else 1
+    if ld < cols:
+        ld = cols
+    return t.data_ptr(), rows, cols, ld if ld > 0 else 1
 
 
 def gemm(A, B, C, alpha: float = 1.0, beta: float = 0.0, mode="auto", select="default",
