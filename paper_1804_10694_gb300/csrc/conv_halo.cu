@@ -563,6 +563,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = false;
           break;
         }
+        __syncwarp();   // lane 0's waits order the other lanes' accesses
         const uint8_t* src = smem + off_stage + st * a.stage_bytes;
         uint8_t* dst = smem + off_slot + hs * a.slot_bytes;
         // four output chunks a thread at a time: all reads first (a store to
