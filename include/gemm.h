@@ -149,10 +149,11 @@ gemm_status gemm_f32_t(int transA, int transB, int64_t M, int64_t N, int64_t K, 
  * thread, computes, copies C back and synchronizes the stream before
  * returning.  Only the M x N (M x K, K x N) elements are copied; padding
  * beyond a row's length in the host buffers is never written.  With
- * page-locked A and C, at least 512 rows, no split-K and the environment
- * variable GEMM_HOST_PANELS (default 16) above 1, B is copied and packed once
- * and row panels of A and C stream through two copy streams while earlier
- * panels compute. */
+ * page-locked A and C, at least 512 rows and no split-K, B is copied and
+ * packed once and row panels of A and C (up to 16, as many as an estimate of
+ * the call's time finds best) stream through two copy streams while earlier
+ * panels compute.  The environment variable GEMM_HOST_PANELS sets the number
+ * of panels; 1 turns them off. */
 gemm_status gemm_f32_host(int64_t M, int64_t N, int64_t K, float alpha, const float* A,
                           int64_t lda, const float* B, int64_t ldb, float beta, float* C,
                           int64_t ldc, gemm_mode mode, gemm_stream_t stream);

@@ -206,7 +206,7 @@ constexpr double kFix0 = 4.0, kFix1 = 0.99;                           // split-K
 constexpr double kSix = 1.6;                                          // six products a chunk
 }  // namespace
 
-int default_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int sms, int max_split) {
+int default_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int sms, int max_split, double* estimate) {
   if (config_count(mode) == 0) return -1;
   const Prec p = prec_of_mode(mode);
   const bool six = mode == GEMM_MODE_BF16X6;
@@ -218,7 +218,7 @@ int default_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int sms, int
   const Tile cands[3] = {{64, 1, kChunk64, kEpi64}, {128, 1, kChunk128, kEpi128}, {256, 2, kChunkPair, kEpiPair}};
   const int splits[] = {1, 2, 3, 4, 6, 8};
   double best = 0.0;
-  int pick = find_config(64, 1, 4, 16);
+  int bn = 64, split = 1, cluster = 1;
   bool have = false;
   for (const Tile& t : cands) {
     if (t.cluster == 2 && sms < 2) continue;
@@ -235,11 +235,12 @@ int default_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int sms, int
       if (!have || est < best) {
         have = true;
         best = est;
-        pick = find_config(t.bn, sk, six && t.cluster == 2 ? 8 : 4, 16, t.cluster);
+        bn = t.bn, split = sk, cluster = t.cluster;
       }
     }
   }
-  return pick;
+  if (estimate) *estimate = best;
+  return find_config(bn, split, six && cluster == 2 ? 8 : 4, 16, cluster);
 }
 
 // Tile width of the gemm without packing for a default BF16X3 plan whose
@@ -1007,17 +1008,16 @@ static cudaError_t copy_rows(float* dst, const float* src, int64_t rows, int64_t
   return cudaMemcpy2DAsync(dst, (size_t)ld * 4, src, (size_t)ld * 4, (size_t)cols * 4, (size_t)rows, kind, s);
 }
 
-// Panels of the host-buffer pipeline (GEMM_HOST_PANELS, default 16; 1 turns
-// the pipeline off).  On 8192^3 with pinned buffers 1/2/4/8/16/32 panels took
-// 7.5/5.7/5.0/4.66/4.53/4.67 ms per call with beta != 0 (4.19/4.25/4.43 ms
-// for 8/16/32 with beta = 0).  The host link carries 211 GB/s host to device
-// alone but 171 + 170 GB/s with both directions busy, so with beta != 0 the
-// floor is about 4.1 ms: the copies back of C panels overlap the copies in.
-static int host_panels() {
+// Panels of the host-buffer pipeline: GEMM_HOST_PANELS of them if set (1 turns
+// the pipeline off), else up to 16, as host_panel_plan finds best.  The host link
+// carries 211 GB/s host to device alone but 171 + 170 GB/s with both directions
+// busy, so the floor of 8192^3 with beta != 0 is about 4.1 ms: the copies back of
+// C panels overlap the copies in.
+static int host_panels_set() {
   static const int n = [] {
     const char* v = std::getenv("GEMM_HOST_PANELS");
-    const int x = v ? std::atoi(v) : 16;
-    return x < 1 ? 1 : (x > 64 ? 64 : x);
+    const int x = v ? std::atoi(v) : 0;
+    return !v ? 0 : x < 1 ? 1 : (x > 64 ? 64 : x);
   }();
   return n;
 }
@@ -1054,16 +1054,27 @@ static int64_t panel_tiles(int64_t tiles_m, int64_t npan, int64_t cl) {
   return ((tiles_m + npan - 1) / npan + cl - 1) / cl * cl;
 }
 
-// Configuration of a plan that the pipelined path runs panel by panel: the best
-// one for a panel, where the one for the whole product has its tiles (-1).  A
-// panel of 256 rows of 4096^3 is 16 pair tiles of the whole product's
-// configuration, on 16 of 76 SM pairs: 80 us behind copies of 45 us.  In 128 x 64
-// tiles it takes the whole chip, and the copies are what the call waits for:
-// 4096^3 with beta != 0 1643 -> 1291 us (same bits).  A product whose own configuration splits
-// K or splits A in the kernel keeps the unpipelined path.
-static gemm_status host_panel_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb, int64_t ldc,
-                                     int* config) {
-  *config = -1;
+// How the pipelined path cuts a product: the number of panels, and the plan's
+// configuration, the best one for a panel (-1: the whole product's own).
+//
+// A call takes B's copy, the panels one after another, each at the pace of the
+// slowest of its copy in, its pack and gemm, and its copy out, and then the last
+// panel's gemm and copy out.  In microseconds: copies at 171 GB/s (B 211), the
+// pack at 5.5 TB/s, the gemm at 0.6 a unit of default_config's estimate and 9 for
+// the two launches.  Within 8 % of what 4 to 16 panels took at 4096^3, 2048^3,
+// 6000 x 1000 x 3000 and 3395 x 800 x 612 but for 4 panels of the first and the
+// last (high and low by 15).  The same 16 panels for all, in the whole product's
+// tiles, left 4096^3 (beta != 0; 16 pair tiles a panel on 76 SM pairs, 80 us
+// behind 50 us of copies) at 1643 us a call: now 1226; 16 panels in their own best
+// tiles took 1277 there, 605 at 2048^3 (now 371), 1160 at 4096^3 with beta = 0
+// (902) and 279 at 3395 x 800 x 612 (144).
+// A product whose own configuration splits K or splits A in the kernel keeps the
+// unpipelined path.
+struct HostPanels {
+  int config = -1, panels = 1;
+};
+static gemm_status host_panel_plan(gemm_mode mode, int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb,
+                                   int64_t ldc, bool reads_c, HostPanels* out) {
   DeviceState* dev;
   int devidx;
   gemm_mode m;
@@ -1074,19 +1085,34 @@ static gemm_status host_panel_config(gemm_mode mode, int64_t M, int64_t N, int64
   const int w = m == GEMM_MODE_F32_SIMT ? -1 : select_config(m, M, N, K, lda, ldb, ldc, GEMM_SELECT_DEFAULT, dev->sms);
   if (w < 0 || !config_get(m, w, &whole) || whole.split_k > 1 || whole.fused) return GEMM_OK;
   const int64_t tiles_m = (M + 127) / 128;
-  const int64_t rows = 128 * panel_tiles(tiles_m, std::min<int64_t>(host_panels(), tiles_m), whole.cluster == 2 ? 2 : 1);
-  const int c = default_config(m, rows, N, K, dev->sms, 1);
-  if (c >= 0 && config_get(m, c, &panel) && (panel.block_n != whole.block_n || panel.cluster != whole.cluster))
-    *config = c;
+  const int set = host_panels_set();
+  double best = 0.0;
+  bool have = false;
+  for (int64_t n = set ? std::min<int64_t>(set, tiles_m) : 1; n <= std::min<int64_t>(set ? set : 16, tiles_m); ++n) {
+    const int64_t rows = 128 * panel_tiles(tiles_m, n, 1), count = (M + rows - 1) / rows;
+    double est = 0.0;
+    const int c = default_config(m, rows, N, K, dev->sms, 1, &est);
+    if (c < 0 || !config_get(m, c, &panel)) continue;
+    const double in = (double)rows * (double)(K + (reads_c ? N : 0)) * 4.0 / 171e3;
+    const double back = (double)rows * (double)N * 4.0 / 171e3;
+    const double gemm = 9.0 + 0.6 * est + (double)rows * (double)K * 8.0 / 5.5e6;
+    const double t = in + (double)(count - 1) * std::max(in, std::max(gemm, back)) + gemm + back;
+    if (!have || t < best) {
+      have = true;
+      best = t;
+      out->panels = (int)n;
+      out->config = panel.block_n != whole.block_n || panel.cluster != whole.cluster ? c : -1;
+    }
+  }
   return GEMM_OK;
 }
 
 // Pipelined path: tensor-core plan without split-K, M spanning >= 2 panels.
-static gemm_status host_gemm_panels(gemm_plan_t p, float alpha, const float* A, const float* B,
+static gemm_status host_gemm_panels(gemm_plan_t p, int panels, float alpha, const float* A, const float* B,
                                     float beta, float* C, cudaStream_t s) {
   const int64_t M = p->M, N = p->N, K = p->K, lda = p->lda, ldb = p->ldb, ldc = p->ldc;
   const int64_t tiles_m = (M + 127) / 128;
-  const int npan = (int)std::min<int64_t>(host_panels(), tiles_m);
+  const int npan = (int)std::min<int64_t>(panels, tiles_m);
   // 128-row tiles per panel; even for a CTA-pair plan (its tiles are 256 rows)
   const int64_t cl = p->launch.cluster == 2 ? 2 : 1;
   const int64_t tiles_per = panel_tiles(tiles_m, npan, cl);
@@ -1177,10 +1203,11 @@ gemm_status host_gemm_impl(int64_t M, int64_t N, int64_t K, float alpha, const f
   if ((st = grow(&t_host.B, &t_host.nB, std::max<size_t>(nB, 1))) != GEMM_OK) return st;
   if ((st = grow(&t_host.C, &t_host.nC, nC)) != GEMM_OK) return st;
   gemm_plan_t p = nullptr;
-  const bool panels = need_ab && host_panels() > 1 && M >= 4 * 128 && page_locked(A) && page_locked(C);
-  int config = -1;
-  if (panels && (st = host_panel_config(mode, M, N, K, lda, ldb, ldc, &config)) != GEMM_OK) return st;
-  if ((st = cached_plan(M, N, K, lda, ldb, ldc, mode, GEMM_SELECT_DEFAULT, s, &p, false, false, config)) != GEMM_OK)
+  const bool panels = need_ab && host_panels_set() != 1 && M >= 4 * 128 && page_locked(A) && page_locked(C);
+  HostPanels cut;
+  if (panels && (st = host_panel_plan(mode, M, N, K, lda, ldb, ldc, beta != 0.0f, &cut)) != GEMM_OK) return st;
+  if ((st = cached_plan(M, N, K, lda, ldb, ldc, mode, GEMM_SELECT_DEFAULT, s, &p, false, false, cut.config)) !=
+      GEMM_OK)
     return st;
   const CachedPlanUse hold(p);
   // (every path below synchronises its streams before returning, so the plan
@@ -1191,7 +1218,7 @@ gemm_status host_gemm_impl(int64_t M, int64_t N, int64_t K, float alpha, const f
     ~NoteUse() { note_use(p, s); }
   } note{p, s};
   if (panels && p->mode != GEMM_MODE_F32_SIMT && p->args.split_k == 1 && !p->unsplit && !p->launch.fused)
-    return host_gemm_panels(p, alpha, A, B, beta, C, s);
+    return host_gemm_panels(p, cut.panels, alpha, A, B, beta, C, s);
   cudaError_t e;
   if (need_ab) {
     if ((e = copy_rows(t_host.A, A, M, K, lda, cudaMemcpyHostToDevice, s)) != cudaSuccess)

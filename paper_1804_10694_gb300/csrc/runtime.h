@@ -73,7 +73,9 @@ int config_count(gemm_mode mode);
 bool config_get(int id, gemm_config* out);
 // The entry as it applies to a mode (false when the id is not one of the mode's).
 bool config_get(gemm_mode mode, int id, gemm_config* out);
-int default_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int sms, int max_split = 8);
+// (estimate: the chosen one's time, in units of about 0.6 microseconds.)
+int default_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int sms, int max_split = 8,
+                   double* estimate = nullptr);
 // Configuration for a new plan under a selection policy (tuning code).
 int select_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb,
                   int64_t ldc, gemm_select sel, int sms);
