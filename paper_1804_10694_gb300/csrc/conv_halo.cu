@@ -400,6 +400,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr int PIECE = 32 * CB * 4;    // bytes of one staged piece
     constexpr int NBUF = 4096 / PIECE;
     constexpr int NP = TW * KN / CB;      // pieces of a unit
+    // The pieces take the buffers in turn, and only those that are stored: the
+    // wait for all but the newest NBUF - 1 stores then covers the buffer's own.
+    // (Counting skipped pieces too, a unit at the right edge handed the buffer
+    // of the newest store to the next unit, unwaited.)
+    static_assert(TW == 1 || KN == CB, "the pieces inside the output come first");
     const int ew = warp - kEpiWarp0;
     const int q = warp & 3;
     const int wg = ew >> 2;
@@ -420,7 +425,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       };
       auto load_old = [&](int i) {        // piece i's old values into its buffer
         if (!piece_in(i)) return;
-        const uint32_t b = (obuf + i) % NBUF;
+        const uint32_t b = (obuf + i) % NBUF;   // (all pieces before it are inside as well)
         if (lane == 0) {
           bulk_wait_read<0>();            // the buffer's last store has read it
           mbar_arrive_expect_tx(cbar(2 * ew + b), PIECE);
@@ -475,9 +480,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         alpha = 1.0f;
       }
       if (a.staged) {
+        uint32_t stored = 0;
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
           if (!piece_in(i)) continue;     // (uniform over the warp)
+          ++stored;
           const uint32_t b = (obuf + i) % NBUF;
           const uint32_t buf = buf0 + b * PIECE;
           if (a.beta != 0.0f) {
@@ -516,7 +523,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           if (a.beta != 0.0f && i + NBUF < NP) load_old(i + NBUF);
         }
-        obuf = (obuf + NP) % NBUF;
+        obuf = (obuf + stored) % NBUF;
         continue;
       }
       // features not a multiple of 4, or a misaligned output: straight stores,

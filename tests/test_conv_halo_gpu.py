@@ -98,3 +98,30 @@ def test_non_finite_pixels(mode):
     assert np.array_equal(np.isfinite(got), np.isfinite(ref))
     ok = np.isfinite(ref).all(axis=-1)
     assert oracle.rel_frob(got[ok], ref[ok]) <= TOL
+
+
+# up to 16 features, several units a CTA, and a last column block whose columns
+# do not fill the tiles of every epilogue warp (one tile in two or none of them)
+RAGGED = [(100, 24, 8, 16, 12, 3, 3), (64, 40, 40, 16, 16, 3, 3), (64, 40, 48, 16, 16, 3, 3), (40, 60, 40, 16, 16, 7, 7),
+          (16, 300, 300, 16, 16, 3, 3)]
+
+
+@pytest.mark.parametrize("mode", ["bf16x3", "tf32x3"])
+@pytest.mark.parametrize("shape", RAGGED)
+@pytest.mark.parametrize("beta", [0.0, 2.0])
+def test_ragged_columns_many_units(mode, shape, beta):
+    """Output pieces that are skipped take no staging buffer: every pixel of
+    the units before and after them is exact, in repeated passes."""
+    n, H, Wd, C, K, R, S = shape
+    x = W.conv_image(n, H, Wd, C, 330, kind="integers")
+    f = W.conv_filter(C, K, 331, kind="integers", R=R, S=S)
+    out0 = W.conv_image(n, H, Wd, K, 332, kind="integers")
+    want = conv.conv_f64(x, f, 1.0, beta, out0).astype(np.float32)
+    plan = pkg.ConvPlan(n, H, Wd, C, K, R, S, mode=mode)
+    dx, df = torch.from_numpy(x).cuda(), torch.from_numpy(f).cuda()
+    for _ in range(5):
+        do = torch.from_numpy(out0.copy()).cuda()
+        plan.execute(dx, df, do, 1.0, beta)
+        assert np.array_equal(do.cpu().numpy(), want)
+    plan.destroy()
+    pkg.device_error()
