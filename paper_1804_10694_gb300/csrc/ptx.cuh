@@ -316,9 +316,10 @@ __device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
-// Orders this thread's generic-proxy writes to shared memory before later
-// async-proxy reads of it (tensor-core operand loads), once the thread's
-// mbarrier arrive is observed by the issuing thread.
+// Orders this thread's generic-proxy accesses to shared memory before later
+// async-proxy ones, once the thread's mbarrier arrive is observed by the issuing
+// thread: its writes before tensor-core operand loads of them, its reads before a
+// TMA copy over them.
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }

@@ -28,7 +28,7 @@
 //
 // Bounded by shared-memory bandwidth (an item of a 128 x 64 tile crosses it four
 // times: copied in, read, written as parts, read by the MMAs, about 850 cycles;
-// 1050 measured) and next by HBM.  50176 x 64 x 576: 72.6 -> 34.5 us a call.
+// 1050 measured) and next by HBM.  50176 x 64 x 576: 72.6 -> 35.7 us a call.
 // Register-staged plain loads instead of TMA took 55 us there (latency),
 // cp.async by the split warps 77 (their proxy fence waits for the copies in
 // flight).
@@ -482,10 +482,13 @@ __global__ void __launch_bounds__(kDirThreads, 1)
           const float uA = max_units<NA>(va), uB = max_units<NB>(vb);
           mA = fmaxf(mA, uA), mB = fmaxf(mB, uB);
           if (pass == 0) {
-            // The stage is free once every lane's values are in registers: the
-            // maxima, which need them all, come before the arrival (an arrival
-            // right behind the reads let the next copy overtake some of them).
-            asm volatile("" ::"f"(uA), "f"(uB) : "memory");
+            // The stage is free once every lane has its values: each lane orders
+            // its reads before the next copy into it (another proxy's writes; an
+            // arrival right behind the reads let the copy overtake some of them).
+            // The fence costs 2 to 3 %.  Given back behind the parts' fence alone,
+            // the stage is late for tall products: 50176 x 64 x 576 40.7 us against
+            // 35.7 (512^3 9.8 against 10.4).
+            fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(sempty(sg));
           }

@@ -105,3 +105,21 @@ def test_turned_tiles(M, N, K, ta, tb):
         for c in (slice(0, 130), slice(130, 200), slice(200, N)):
             assert oracle.rel_frob(got[r, c], want[r, c]) <= TOL, (r, c)
     pkg.device_error()
+
+
+@pytest.mark.parametrize("M,N,K", [(50176, 64, 576), (100000, 32, 512), (1060, 1060, 1060)])
+def test_stage_reuse(M, N, K):
+    """Long runs of items through the staging ring, pass after pass: a copy
+    that overtook a split warp's reads of the item before would change bits."""
+    g = torch.Generator(device="cuda").manual_seed(530)
+    a, b = (torch.empty(s, device="cuda").uniform_(-1, 1, generator=g) for s in ((M, K), (K, N)))
+    ab = torch.full((M * K + 1,), float("nan"), device="cuda")
+    ab[1:] = a.view(-1)
+    want, got = torch.empty(M, N, device="cuda"), torch.empty(M, N, device="cuda")
+    s = torch.cuda.current_stream().cuda_stream
+    pkg.gemm_f32_ex(M, N, K, 1.0, ab.data_ptr() + 4, K, b.data_ptr(), N, 0.0, want.data_ptr(), N, "bf16x3", "default", s)
+    for _ in range(20):
+        got.fill_(float("nan"))
+        pkg.gemm(a, b, got, mode="bf16x3")
+        assert torch.equal(got.view(torch.int32), want.view(torch.int32))
+    pkg.device_error()
