@@ -258,9 +258,13 @@ int default_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int sms, int
 // 22.6), 60000 x 256 x 576 (131 against 144), 700 x 900 x 1300 (21.8 against
 // 24.6).  1060^3 took 29.3 packed, 36 in two waves of tiles here and 22.9 in one,
 // its last rows in turned tiles (direct_grid); 1088^3 26.6 -> 21.3.
-// A split-K configuration gives way (to the unsplit tile, for operands that TMA
-// cannot load) only where M, N and K are multiples of 4, that is where every
-// tight layout can be loaded.
+// A split-K configuration gives way (to the unsplit tile, for operands that start
+// off a 16-byte boundary) only where M, N and K are multiples of 4.  Plans whose
+// leading dimensions are not never come here: TMA could load no operand of theirs
+// (512^3 with rows of 1001 floats 15.2 us unsplit, 13.8 in the split-K configuration
+// it keeps).  An operand that starts off a 16-byte boundary is seen only at the
+// call, whose bits are to be those of any other: the unsplit tile it then runs
+// took 15.2 us at 512^3 and 18.8 at 768^3, the split ones 13.8 and 17.2.
 static int direct_tile(const gemm_config& c, int64_t M, int64_t N, int64_t K, int sms) {
   const int64_t chunks = (K + 63) / 64, items = (K + 31) / 32, tm = (M + 127) / 128;
   if (c.split_k > 1 && ((M | N | K) & 3) != 0) return 0;
@@ -492,7 +496,8 @@ gemm_status plan_create_impl(int64_t M, int64_t N, int64_t K, int64_t lda, int64
   }
   if (!config_get(m, config_id, &p->cfg))
     return fail(GEMM_ERR_INVALID_ARG, "configuration id %d out of range for mode %d", config_id, (int)m);
-  if (default_choice && m == GEMM_MODE_BF16X3 && conv_image_elems < 0 && !comp && p->cfg.cluster == 1) {
+  if (default_choice && m == GEMM_MODE_BF16X3 && conv_image_elems < 0 && !comp && p->cfg.cluster == 1 &&
+      lda % 4 == 0 && ldb % 4 == 0) {
     p->direct = direct_tile(p->cfg, M, N, K, dev->sms);
     if (p->direct && p->cfg.split_k > 1) {
       config_id = find_config(64, 1, p->cfg.kb, p->cfg.group_m);   // the same sums, unsplit
@@ -719,8 +724,8 @@ gemm_status plan_execute_impl(gemm_plan_t p, float alpha, const float* A, const 
   const bool prof = p->prof_n < p->prof_max;
   cudaEvent_t* ev = prof ? &p->prof_events[4 * p->prof_n] : nullptr;
   if (prof) cudaEventRecord(ev[0], s);
-  auto rows16 = [](const float* X, int64_t ld) { return ld % 4 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0; };
-  if (p->direct && rows16(A, p->lda) && rows16(B, p->ldb)) {
+  auto aligned = [](const float* X) { return reinterpret_cast<uintptr_t>(X) % 16 == 0; };
+  if (p->direct && aligned(A) && aligned(B)) {
     DirectArgs d{};
     d.A = A, d.B = B, d.C = C;
     d.lda = p->lda, d.ldb = p->ldb, d.ldc = p->ldc;

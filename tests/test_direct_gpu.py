@@ -123,3 +123,25 @@ def test_stage_reuse(M, N, K):
         pkg.gemm(a, b, got, mode="bf16x3")
         assert torch.equal(got.view(torch.int32), want.view(torch.int32))
     pkg.device_error()
+
+
+@pytest.mark.parametrize("M,N,K,lda,ldb", [(512, 512, 512, 513, 512), (512, 512, 512, 512, 1001), (384, 384, 384, 385, 390)])
+def test_rows_off_16_bytes_keep_their_configuration(M, N, K, lda, ldb):
+    """Leading dimensions that are not multiples of 4 rule the kernel out for
+    every call of the plan, which then runs what it would without it: the
+    default split-K configuration, its bits and its workspace."""
+    c = pkg.config_default("bf16x3", M, N, K)
+    assert pkg.config_get("bf16x3", c)["split_k"] > 1
+    A, B, C0 = W._with_ld(W.uniform(M, K, 540), lda, np.nan), W._with_ld(W.uniform(K, N, 541), ldb, np.nan), W.uniform(M, N, 542)
+    a, b = (torch.from_numpy(x).cuda() for x in (A, B))
+    out, info = [], []
+    for config in (None, c):
+        plan = pkg.Plan(M, N, K, lda, ldb, N, mode="bf16x3", config_id=config)
+        info.append(plan.info())
+        d = torch.from_numpy(C0.copy()).cuda()
+        plan.execute_ptrs(1.5, a.data_ptr(), b.data_ptr(), 0.5, d.data_ptr())
+        out.append(d.cpu().numpy())
+        plan.destroy()
+    assert info[0] == info[1] and info[0]["config_id"] == c
+    assert np.array_equal(out[0].view(np.uint32), out[1].view(np.uint32))
+    assert oracle.rel_frob(out[0], oracle.gemm_f64(M, N, K, 1.5, A, B, 0.5, C0)) <= TOL
