@@ -329,6 +329,11 @@ static gemm_status encode_planes(CUtensorMap* map, Prec p, void* base, int64_t r
   return GEMM_OK;
 }
 
+// Whether the rows of an FP32 operand, ld floats apart, fit a tensor map: its
+// strides are multiples of 16 bytes, and below 2^40 (a single row's leading
+// dimension may be anything).
+static bool tma_rows(int64_t rows, int64_t ld) { return ld % 4 == 0 && ld <= ((int64_t(1) << 38) - 1) / rows; }
+
 // An FP32 operand itself, rows x cols stored row-major: boxes of box_r rows x
 // 32 columns (128 bytes), 128-byte swizzle, zero fill outside.  Needs a 16-byte
 // aligned base and ld % 4 == 0.
@@ -497,7 +502,7 @@ gemm_status plan_create_impl(int64_t M, int64_t N, int64_t K, int64_t lda, int64
   if (!config_get(m, config_id, &p->cfg))
     return fail(GEMM_ERR_INVALID_ARG, "configuration id %d out of range for mode %d", config_id, (int)m);
   if (default_choice && m == GEMM_MODE_BF16X3 && conv_image_elems < 0 && !comp && p->cfg.cluster == 1 &&
-      lda % 4 == 0 && ldb % 4 == 0) {
+      tma_rows(transA ? K : M, lda) && tma_rows(transB ? N : K, ldb)) {
     p->direct = direct_tile(p->cfg, M, N, K, dev->sms);
     if (p->direct && p->cfg.split_k > 1) {
       config_id = find_config(64, 1, p->cfg.kb, p->cfg.group_m);   // the same sums, unsplit

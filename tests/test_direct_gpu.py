@@ -145,3 +145,21 @@ def test_rows_off_16_bytes_keep_their_configuration(M, N, K, lda, ldb):
     assert info[0] == info[1] and info[0]["config_id"] == c
     assert np.array_equal(out[0].view(np.uint32), out[1].view(np.uint32))
     assert oracle.rel_frob(out[0], oracle.gemm_f64(M, N, K, 1.5, A, B, 0.5, C0)) <= TOL
+
+
+@pytest.mark.parametrize("ta,tb,M,N,K", [(0, 0, 1, 64, 64), (0, 0, 64, 64, 1), (1, 0, 64, 64, 1), (0, 1, 64, 1, 64)])
+def test_single_rows_with_any_leading_dimension(ta, tb, M, N, K):
+    """A single stored row's leading dimension is never used: one past a
+    tensor map's strides runs the packed path, with the same bits."""
+    A, B = W.uniform(M, K, 550), W.uniform(K, N, 551)
+    a, b = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (A.T if ta else A, B.T if tb else B))
+    far = [2 ** 38 if x.shape[0] == 1 else x.shape[1] for x in (a, b)]
+    out = []
+    for lda, ldb in ((a.shape[1], b.shape[1]), far):
+        c = torch.zeros(M, N, device="cuda")
+        pkg.gemm_f32_t(ta, tb, M, N, K, 1.5, a.data_ptr(), lda, b.data_ptr(), ldb, 0.0, c.data_ptr(), N, "bf16x3", "default",
+                       torch.cuda.current_stream().cuda_stream)
+        out.append(c.cpu().numpy())
+    assert 2 ** 38 in far
+    assert np.array_equal(out[0].view(np.uint32), out[1].view(np.uint32))
+    assert oracle.rel_frob(out[0], oracle.gemm_f64(M, N, K, 1.5, A, B, 0.0, None)) <= TOL
