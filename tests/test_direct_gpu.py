@@ -163,3 +163,20 @@ def test_single_rows_with_any_leading_dimension(ta, tb, M, N, K):
     assert 2 ** 38 in far
     assert np.array_equal(out[0].view(np.uint32), out[1].view(np.uint32))
     assert oracle.rel_frob(out[0], oracle.gemm_f64(M, N, K, 1.5, A, B, 0.0, None)) <= TOL
+
+
+@pytest.mark.parametrize("n", [384, 448, 512, 640])
+def test_unsplit_sums_are_the_split_ones(n):
+    """In place of a split-K configuration whose parts are one fold each, the
+    kernel folds at the parts' ends: without alpha and beta the sums of the
+    parts in their order, the same bits."""
+    c = pkg.config_default("bf16x3", n, n, n)
+    cfg = pkg.config_get("bf16x3", c)
+    chunks = (n + 63) // 64
+    assert cfg["split_k"] > 1 and -(-chunks // cfg["split_k"]) <= cfg["kb"]
+    a, b = (torch.from_numpy(W.uniform(n, n, s)).cuda() for s in (560, 561))
+    got = pkg.gemm(a, b, torch.empty(n, n, device="cuda"), mode="bf16x3")
+    plan = pkg.Plan(n, n, n, mode="bf16x3", config_id=c)
+    want = plan.execute(a, b, torch.empty(n, n, device="cuda"))
+    assert torch.equal(got.view(torch.int32), want.view(torch.int32))
+    plan.destroy()
