@@ -1119,7 +1119,12 @@ static gemm_status host_panel_plan(gemm_mode mode, int64_t M, int64_t N, int64_t
       have = true;
       best = t;
       out->panels = (int)n;
-      out->config = panel.block_n != whole.block_n || panel.cluster != whole.cluster ? c : -1;
+      // (never with longer folds than the whole product's: BF16X6 folds its pair
+      // tiles half as often by default, and panels of 1202 x 5016 x 1057 on them had
+      // an error of 3.9e-7 where the product on device buffers has 2.0e-7)
+      out->config = panel.block_n != whole.block_n || panel.cluster != whole.cluster
+                        ? find_config(panel.block_n, 1, std::min(panel.kb, whole.kb), panel.group_m, panel.cluster)
+                        : -1;
     }
   }
   return GEMM_OK;

@@ -22,3 +22,21 @@ def test_panels_match_device_buffers(mode, M, N, K, beta):
     got = pkg.gemm_host(A, B, C, 1.5, beta, mode=mode)
     assert torch.equal(got.view(torch.int32), want.view(torch.int32))
     pkg.device_error()
+
+
+@pytest.mark.parametrize("M,N,K", [(1202, 5016, 1057), (2048, 2048, 2048), (4099, 2050, 1000)])
+@pytest.mark.parametrize("beta", [0.0, 0.5])
+def test_six_product_panels_are_as_accurate(M, N, K, beta):
+    """BF16X6, whose pair tiles fold half as often as the single ones by
+    default: panels on pairs of a product that runs on single tiles keep its
+    folds (the first shape: the same bits), and none is less accurate."""
+    g = torch.Generator().manual_seed(710)
+    A, B, C = (torch.empty(s).uniform_(-1, 1, generator=g).pin_memory() for s in ((M, K), (K, N), (M, N)))
+    a, b, c = A.cuda(), B.cuda(), C.cuda()
+    exact = 1.5 * (a.double() @ b.double()) + beta * c.double()
+    want = pkg.gemm(a, b, c, 1.5, beta, mode="bf16x6")
+    got = pkg.gemm_host(A, B, C, 1.5, beta, mode="bf16x6").cuda()
+    assert (got.double() - exact).norm() <= (want.double() - exact).norm()
+    if (M, N, K) == (1202, 5016, 1057):
+        assert torch.equal(got.view(torch.int32), want.view(torch.int32))
+    pkg.device_error()
