@@ -75,19 +75,6 @@ inline int chunk_stride(int px, bool tf32) {
   return (px * 16 + 127) / 128 * 128 + 128 / chunks_of(tf32);
 }
 
-__device__ __forceinline__ unsigned cvt2_bf16(float lo_half, float hi_half) {
-  unsigned d;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi_half), "f"(lo_half));
-  return d;
-}
-
-// Unswizzled K-major operand: 8-row x 16-byte core matrices, `lbo` bytes from
-// one 16-byte K chunk to the next, `sbo` from one group of 8 rows to the next.
-__device__ __forceinline__ uint64_t sdesc_k_plain(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  return static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4) | (static_cast<uint64_t>(lbo >> 4) << 16) |
-         (static_cast<uint64_t>(sbo >> 4) << 32) | (static_cast<uint64_t>(1) << 46);
-}
-
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, float4 v) {
   asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
                : "memory");
@@ -99,38 +86,23 @@ __device__ __forceinline__ float4 ld_shared_v4(uint32_t addr) {
 }
 
 // One 16-byte chunk of hi and of lo parts from its FP32 values (finite: none
-// of them is Inf or NaN, so that pairs convert in one instruction; the bits
-// are those of split_bf16 / split_tf32 either way).
+// of them is Inf or NaN; the bits are those of split_bf16 / split_tf32).
 template <bool TF32>
 __device__ __forceinline__ void split_chunk(const float* x, bool finite, uint4& hv, uint4& lv) {
-  unsigned h[4], l[4];
   if constexpr (TF32) {
     (void)finite;
+    unsigned h[4], l[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       float a, b;
       split_tf32(x[k], a, b);
       h[k] = __float_as_uint(a), l[k] = __float_as_uint(b);
     }
-  } else if (finite) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      h[k] = cvt2_bf16(x[2 * k], x[2 * k + 1]);
-      l[k] = cvt2_bf16(__fsub_rn(x[2 * k], __uint_as_float(h[k] << 16)),
-                       __fsub_rn(x[2 * k + 1], __uint_as_float(h[k] & 0xFFFF0000u)));
-    }
+    hv = make_uint4(h[0], h[1], h[2], h[3]);
+    lv = make_uint4(l[0], l[1], l[2], l[3]);
   } else {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const HiLoBf16 s0 = split_bf16(x[2 * k]), s1 = split_bf16(x[2 * k + 1]);
-      h[k] = static_cast<unsigned>(__bfloat16_as_ushort(s0.hi)) |
-             (static_cast<unsigned>(__bfloat16_as_ushort(s1.hi)) << 16);
-      l[k] = static_cast<unsigned>(__bfloat16_as_ushort(s0.lo)) |
-             (static_cast<unsigned>(__bfloat16_as_ushort(s1.lo)) << 16);
-    }
+    split_chunk_bf16(x, finite, hv, lv);
   }
-  hv = make_uint4(h[0], h[1], h[2], h[3]);
-  lv = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
 // Position of unit u: output-feature block fastest, then column block, row
@@ -303,7 +275,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       constexpr uint32_t idesc1 = idesc_f32acc(TF32, 128, KN);
       const int is = warp >> 1;
       // descriptors move by adding 16-byte units to their address field
-      const uint64_t slot0 = sdesc_k_plain(sbase + off_slot + is * 128, a.chb, a.bw * 16);
+      const uint64_t slot0 = sdesc_plain(sbase + off_slot + is * 128, a.chb, a.bw * 16);
       const uint64_t w0 = sdesc_k_sw128(sbase);
       const uint32_t slot_units = a.slot_bytes >> 4, sub_units = a.chb >> 3, lo_units = (NJ * a.chb) >> 4;
       const uint32_t row_units = a.bw - a.S;   // from a filter row's last column to the next row's first

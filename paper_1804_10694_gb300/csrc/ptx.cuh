@@ -437,6 +437,14 @@ __device__ __forceinline__ uint64_t sdesc_k(uint32_t saddr) {
   return SW == 128 ? sdesc_k_sw128(saddr) : sdesc_k_sw64(saddr);
 }
 
+// Unswizzled operand: 8 x 16-byte core matrices, `lbo` bytes from one to the
+// next along the leading dimension (K-major: 16-byte chunks of K) and `sbo` along
+// the stride dimension (K-major: groups of 8 rows).
+__device__ __forceinline__ uint64_t sdesc_plain(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+  return static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4) | (static_cast<uint64_t>(lbo >> 4) << 16) |
+         (static_cast<uint64_t>(sbo >> 4) << 32) | (static_cast<uint64_t>(1) << 46);
+}
+
 // Instruction descriptor for kind::f16 (bf16 operands) / kind::tf32 with FP32
 // accumulation, dense, both operands K-major.
 //   bits 4-5 D format (1 = F32); bits 7-9 / 10-12 A / B format (1 = BF16, 2 = TF32)

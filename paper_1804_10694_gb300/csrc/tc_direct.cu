@@ -86,10 +86,6 @@ struct DirCfg {
   static_assert(SMEM <= 231424 && ITEM % 1024 == 0, "shared memory");
 };
 
-__device__ __forceinline__ uint64_t desc_plain(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  return static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4) | (static_cast<uint64_t>(lbo >> 4) << 16) |
-         (static_cast<uint64_t>(sbo >> 4) << 32) | (static_cast<uint64_t>(1) << 46);
-}
 // A staged operand is a run of 128-byte rows of 32 neighbouring stored values
 // (K-major: the operand's rows; MN-major: piece by piece of 32 rows, its k), in
 // the 128-byte swizzle.  A split thread's unit n is the quarter row t + 128 n:
@@ -323,9 +319,9 @@ __global__ void __launch_bounds__(kDirThreads, 1)
       auto set_roles = [&](bool turned) {
         const bool mnA = mn_a(turned), mnB = mn_b(turned);
         idesc = idesc_f32acc(false, 128, BN) | (mnA ? 1u << 15 : 0u) | (mnB ? 1u << 16 : 0u);
-        dA0 = mnA ? desc_plain(s0, 128, kChbMn) : desc_plain(s0, kChbK, 128);
-        dB0 = mnB ? desc_plain(s0 + 2 * Cfg::A_PLANE, 128, kChbMn)
-                  : desc_plain(s0 + 2 * Cfg::A_PLANE, Cfg::CHB_BK, 128);
+        dA0 = mnA ? sdesc_plain(s0, 128, kChbMn) : sdesc_plain(s0, kChbK, 128);
+        dB0 = mnB ? sdesc_plain(s0 + 2 * Cfg::A_PLANE, 128, kChbMn)
+                  : sdesc_plain(s0 + 2 * Cfg::A_PLANE, Cfg::CHB_BK, 128);
         stepA = (mnA ? 256 : 2 * kChbK) >> 4, stepB = (mnB ? 256 : 2 * Cfg::CHB_BK) >> 4;
         // the packed kernel's products in its order: lo*hi, hi*lo, hi*hi (of A and B)
         a1 = turned ? 0 : loA, b1 = turned ? loB : 0, a2 = turned ? loA : 0, b2 = turned ? 0 : loB;
