@@ -855,12 +855,10 @@ struct CacheKey {
   int dev;
   int64_t M, N, K, lda, ldb, ldc;
   int mode, sel, trans;
-  int config;               // configuration id, or -1: by sel
   uintptr_t stream;
   bool operator<(const CacheKey& o) const {
-    return std::tie(dev, M, N, K, lda, ldb, ldc, mode, sel, trans, config, stream) <
-           std::tie(o.dev, o.M, o.N, o.K, o.lda, o.ldb, o.ldc, o.mode, o.sel, o.trans, o.config,
-                    o.stream);
+    return std::tie(dev, M, N, K, lda, ldb, ldc, mode, sel, trans, stream) <
+           std::tie(o.dev, o.M, o.N, o.K, o.lda, o.ldb, o.ldc, o.mode, o.sel, o.trans, o.stream);
   }
   bool operator==(const CacheKey& o) const { return !(*this < o) && !(o < *this); }
 };
@@ -901,11 +899,11 @@ static bool stream_capturing(cudaStream_t s) {
 
 gemm_status cached_plan(int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb, int64_t ldc,
                         gemm_mode mode, gemm_select sel, cudaStream_t s, gemm_plan_t* out,
-                        bool transA, bool transB, int config = -1) {
+                        bool transA, bool transB) {
   int dev = 0;
   cudaGetDevice(&dev);
   CacheKey key{dev, M, N, K, lda, ldb, ldc, (int)mode, (int)sel, (transA ? 1 : 0) | (transB ? 2 : 0),
-               config, reinterpret_cast<uintptr_t>(s)};
+               reinterpret_cast<uintptr_t>(s)};
   // (the capture status is read first: while this thread's stream is being
   // captured, no event of an eager execution is queried)
   const bool capturing = stream_capturing(s);
@@ -926,7 +924,7 @@ gemm_status cached_plan(int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ld
                 "no cached plan for this shape and stream while the stream is being captured: "
                 "call once before the capture, or capture an explicit plan (gemm_plan_create)");
   gemm_plan_t p = nullptr;
-  gemm_status st = plan_create_impl(M, N, K, lda, ldb, ldc, mode, config, sel, &p, transA, transB);
+  gemm_status st = plan_create_impl(M, N, K, lda, ldb, ldc, mode, -1, sel, &p, transA, transB);
   if (st != GEMM_OK) return st;
   cudaError_t e = cudaEventCreateWithFlags(&p->last_use, cudaEventDisableTiming);
   if (e != cudaSuccess) {
@@ -1072,8 +1070,8 @@ static int64_t panel_tiles(int64_t tiles_m, int64_t npan, int64_t cl) {
   return ((tiles_m + npan - 1) / npan + cl - 1) / cl * cl;
 }
 
-// How the pipelined path cuts a product: the number of panels, and the plan's
-// configuration, the best one for a panel (-1: the whole product's own).
+// How the pipelined path cuts a product: the number of panels, and their tiles, the
+// best ones for a panel.
 //
 // A call takes B's copy, the panels one after another, each at the pace of the
 // slowest of its copy in, its pack and gemm, and its copy out, and then the last
@@ -1086,22 +1084,15 @@ static int64_t panel_tiles(int64_t tiles_m, int64_t npan, int64_t cl) {
 // behind 50 us of copies) at 1643 us a call: now 1226; 16 panels in their own best
 // tiles took 1277 there, 605 at 2048^3 (now 371), 1160 at 4096^3 with beta = 0
 // (902) and 279 at 3395 x 800 x 612 (144).
-// A product whose own configuration splits K or splits A in the kernel keeps the
-// unpipelined path.
+// The panels run in the product's own plan, with its planes: one plan a shape,
+// whichever entry points it is called through.
 struct HostPanels {
-  int config = -1, panels = 1;
+  int panels;
+  gemm_config tile;
 };
-static gemm_status host_panel_plan(gemm_mode mode, int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb,
-                                   int64_t ldc, bool reads_c, HostPanels* out) {
-  DeviceState* dev;
-  int devidx;
-  gemm_mode m;
-  gemm_status st = device_state(&dev, &devidx);
-  if (st == GEMM_OK) st = resolve_mode(mode, *dev, &m);
-  if (st != GEMM_OK) return st;
-  gemm_config whole, panel;
-  const int w = m == GEMM_MODE_F32_SIMT ? -1 : select_config(m, M, N, K, lda, ldb, ldc, GEMM_SELECT_DEFAULT, dev->sms);
-  if (w < 0 || !config_get(m, w, &whole) || whole.split_k > 1 || whole.fused) return GEMM_OK;
+static HostPanels host_panel_plan(gemm_plan_t p, bool reads_c) {
+  const int64_t M = p->M, N = p->N, K = p->K;
+  HostPanels out{1, p->cfg};
   const int64_t tiles_m = (M + 127) / 128;
   const int set = host_panels_set();
   double best = 0.0;
@@ -1109,8 +1100,9 @@ static gemm_status host_panel_plan(gemm_mode mode, int64_t M, int64_t N, int64_t
   for (int64_t n = set ? std::min<int64_t>(set, tiles_m) : 1; n <= std::min<int64_t>(set ? set : 16, tiles_m); ++n) {
     const int64_t rows = 128 * panel_tiles(tiles_m, n, 1), count = (M + rows - 1) / rows;
     double est = 0.0;
-    const int c = default_config(m, rows, N, K, dev->sms, 1, &est);
-    if (c < 0 || !config_get(m, c, &panel)) continue;
+    gemm_config panel;
+    const int c = default_config(p->mode, rows, N, K, p->sms, 1, &est);
+    if (c < 0 || !config_get(p->mode, c, &panel)) continue;
     const double in = (double)rows * (double)(K + (reads_c ? N : 0)) * 4.0 / 171e3;
     const double back = (double)rows * (double)N * 4.0 / 171e3;
     const double gemm = 9.0 + 0.6 * est + (double)rows * (double)K * 8.0 / 5.5e6;
@@ -1118,29 +1110,54 @@ static gemm_status host_panel_plan(gemm_mode mode, int64_t M, int64_t N, int64_t
     if (!have || t < best) {
       have = true;
       best = t;
-      out->panels = (int)n;
+      out.panels = (int)n;
+      out.tile = panel;
       // (never with longer folds than the whole product's: BF16X6 folds its pair
       // tiles half as often by default, and panels of 1202 x 5016 x 1057 on them had
       // an error of 3.9e-7 where the product on device buffers has 2.0e-7)
-      out->config = panel.block_n != whole.block_n || panel.cluster != whole.cluster
-                        ? find_config(panel.block_n, 1, std::min(panel.kb, whole.kb), panel.group_m, panel.cluster)
-                        : -1;
+      out.tile.kb = std::min(panel.kb, p->cfg.kb);
     }
   }
-  return GEMM_OK;
+  return out;
+}
+
+// Plan p's launch, unsplit, in the tiles of configuration c: what differs from the
+// plan's own but for the number of row tiles, which is the panel's.
+struct PanelLaunch {
+  TcArgs args;
+  TcLaunch launch;
+  CUtensorMap tmB;
+  int max_pairs;
+};
+static gemm_status panel_launch(gemm_plan_t p, const gemm_config& c, PanelLaunch* out) {
+  out->args = p->args, out->launch = p->launch, out->tmB = p->tmB, out->max_pairs = p->max_pairs;
+  const int cluster = c.cluster == 2 ? 2 : 1, sw = tc_chunk_bytes(c.block_n);
+  out->args.tiles_n = (int)((p->N + c.block_n - 1) / c.block_n);
+  out->args.kb = std::max(1, std::min(c.kb, kMaxFoldChunks)) * (128 / sw);
+  out->args.group_m = std::max(1, c.group_m / cluster);
+  if (c.block_n == p->cfg.block_n && c.cluster == p->cfg.cluster) return GEMM_OK;
+  out->launch.bn = c.block_n;
+  out->launch.cluster = cluster;
+  cudaError_t e = cluster == 2 ? tc_pair_prepare(c.block_n, p->prec, &out->max_pairs)
+                               : tc_prepare(c.block_n, p->prec, false);
+  if (e != cudaSuccess) return cuda_fail(e, "kernel attribute");
+  return encode_planes(&out->tmB, p->prec, p->planesB, p->N, p->K, p->pitch, c.block_n / cluster, sw);
 }
 
 // Pipelined path: tensor-core plan without split-K, M spanning >= 2 panels.
-static gemm_status host_gemm_panels(gemm_plan_t p, int panels, float alpha, const float* A, const float* B,
+static gemm_status host_gemm_panels(gemm_plan_t p, float alpha, const float* A, const float* B,
                                     float beta, float* C, cudaStream_t s) {
+  const HostPanels cut = host_panel_plan(p, beta != 0.0f);
+  PanelLaunch pl;
+  gemm_status st = panel_launch(p, cut.tile, &pl);
+  if (st != GEMM_OK) return st;
   const int64_t M = p->M, N = p->N, K = p->K, lda = p->lda, ldb = p->ldb, ldc = p->ldc;
   const int64_t tiles_m = (M + 127) / 128;
-  const int npan = (int)std::min<int64_t>(panels, tiles_m);
-  // 128-row tiles per panel; even for a CTA-pair plan (its tiles are 256 rows)
-  const int64_t cl = p->launch.cluster == 2 ? 2 : 1;
+  const int npan = (int)std::min<int64_t>(cut.panels, tiles_m);
+  // 128-row tiles per panel; even for CTA pairs (their tiles are 256 rows)
+  const int64_t cl = pl.launch.cluster == 2 ? 2 : 1;
   const int64_t tiles_per = panel_tiles(tiles_m, npan, cl);
-  gemm_status st = host_streams(2 + 2 * npan);
-  if (st != GEMM_OK) return st;
+  if ((st = host_streams(2 + 2 * npan)) != GEMM_OK) return st;
   cudaEvent_t* ev = t_host.ev.data();
   cudaError_t e;
   // the copies start after whatever the caller queued on s
@@ -1177,7 +1194,7 @@ static gemm_status host_gemm_panels(gemm_plan_t p, int panels, float alpha, cons
                                     static_cast<char*>(p->planesA) + r0 * p->pitch * prec_elem_bytes(p->prec),
                                     M * p->pitch, p->pitch, p->sms, s)))
       return cuda_fail(e, "pack A panel");
-    TcArgs a = p->args;
+    TcArgs a = pl.args;
     a.alpha = alpha;
     a.beta = beta;
     a.C = t_host.C;
@@ -1188,13 +1205,13 @@ static gemm_status host_gemm_panels(gemm_plan_t p, int panels, float alpha, cons
     a.readyB = p->cntB;
     // the maxima are read by every panel's gemm: only the last one clears them
     if (t1 < tiles_m) a.state_words = 0;
-    a.tiles_m = (int)((t1 - t0 + cl - 1) / cl);   // in the plan's tile height
+    a.tiles_m = (int)((t1 - t0 + cl - 1) / cl);   // in the tiles' height
     a.num_tiles = a.tiles_m * a.tiles_n;
     a.num_units = a.num_tiles;   // split_k == 1
     a.group_m = std::max(1, std::min(a.group_m, a.tiles_m));
-    TcLaunch l = p->launch;
-    l.grid = cl == 2 ? 2 * std::min(a.num_units, p->max_pairs) : std::min(a.num_units, p->sms);
-    if ((e = tc_gemm_launch(l, p->tmA, p->tmB, a, s)) || (e = cudaEventRecord(ev[2 + npan + i], s)) ||
+    TcLaunch l = pl.launch;
+    l.grid = cl == 2 ? 2 * std::min(a.num_units, pl.max_pairs) : std::min(a.num_units, p->sms);
+    if ((e = tc_gemm_launch(l, p->tmA, pl.tmB, a, s)) || (e = cudaEventRecord(ev[2 + npan + i], s)) ||
         (e = cudaStreamWaitEvent(t_host.d2h, ev[2 + npan + i], 0)) ||
         (e = copy_rows(C + r0 * ldc, t_host.C + r0 * ldc, r1 - r0, N, ldc, cudaMemcpyDeviceToHost,
                        t_host.d2h)))
@@ -1226,11 +1243,7 @@ gemm_status host_gemm_impl(int64_t M, int64_t N, int64_t K, float alpha, const f
   if ((st = grow(&t_host.B, &t_host.nB, std::max<size_t>(nB, 1))) != GEMM_OK) return st;
   if ((st = grow(&t_host.C, &t_host.nC, nC)) != GEMM_OK) return st;
   gemm_plan_t p = nullptr;
-  const bool panels = need_ab && host_panels_set() != 1 && M >= 4 * 128 && page_locked(A) && page_locked(C);
-  HostPanels cut;
-  if (panels && (st = host_panel_plan(mode, M, N, K, lda, ldb, ldc, beta != 0.0f, &cut)) != GEMM_OK) return st;
-  if ((st = cached_plan(M, N, K, lda, ldb, ldc, mode, GEMM_SELECT_DEFAULT, s, &p, false, false, cut.config)) !=
-      GEMM_OK)
+  if ((st = cached_plan(M, N, K, lda, ldb, ldc, mode, GEMM_SELECT_DEFAULT, s, &p, false, false)) != GEMM_OK)
     return st;
   const CachedPlanUse hold(p);
   // (every path below synchronises its streams before returning, so the plan
@@ -1240,8 +1253,9 @@ gemm_status host_gemm_impl(int64_t M, int64_t N, int64_t K, float alpha, const f
     cudaStream_t s;
     ~NoteUse() { note_use(p, s); }
   } note{p, s};
-  if (panels && p->mode != GEMM_MODE_F32_SIMT && p->args.split_k == 1 && !p->unsplit && !p->launch.fused)
-    return host_gemm_panels(p, cut.panels, alpha, A, B, beta, C, s);
+  if (need_ab && p->mode != GEMM_MODE_F32_SIMT && p->args.split_k == 1 && !p->unsplit && !p->launch.fused &&
+      host_panels_set() != 1 && M >= 4 * 128 && page_locked(A) && page_locked(C))
+    return host_gemm_panels(p, alpha, A, B, beta, C, s);
   cudaError_t e;
   if (need_ab) {
     if ((e = copy_rows(t_host.A, A, M, K, lda, cudaMemcpyHostToDevice, s)) != cudaSuccess)

@@ -40,3 +40,28 @@ def test_six_product_panels_are_as_accurate(M, N, K, beta):
     if (M, N, K) == (1202, 5016, 1057):
         assert torch.equal(got.view(torch.int32), want.view(torch.int32))
     pkg.device_error()
+
+
+def test_host_calls_use_the_shape_s_own_plan():
+    """Panels in other tiles than the whole product's take no plan of their
+    own: a shape that went through host buffers can be captured on device
+    buffers, and further host calls allocate nothing on the device."""
+    n = 2048
+    g = torch.Generator().manual_seed(720)
+    A, B, C = (torch.empty(n, n).uniform_(-1, 1, generator=g).pin_memory() for _ in range(3))
+    a, b, c = A.cuda(), B.cuda(), C.cuda()
+    want = 1.5 * (a.double() @ b.double()) + 0.5 * c.double()
+    s, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    for beta in (0.0, 0.5):
+        pkg.gemm_host(A, B, C.clone().pin_memory(), 1.5, beta, mode="bf16x3", stream=s)
+    free = torch.cuda.mem_get_info()[0]
+    for beta in (0.5, 0.0, 0.5):
+        pkg.gemm_host(A, B, C.clone().pin_memory(), 1.5, beta, mode="bf16x3", stream=s)
+    assert torch.cuda.mem_get_info()[0] == free
+    with torch.cuda.graph(graph, stream=s):
+        pkg.gemm(a, b, c, 1.5, 0.5, mode="bf16x3", stream=s)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert (c.double() - want).norm() <= 1e-5 * want.norm()
+    pkg.device_error()
