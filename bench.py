@@ -337,9 +337,10 @@ def _median_ms(fn, reps, stream):
 def other_workloads(model_path: str | None):
     """Secondary measurements on the other workloads (outside the timed
     region; device-filled uniform[-1, 1] data, median of CUDA-event timings):
-    the square sweep in every mode, the conv-as-gemm shapes with the
-    heuristic, the cost model's pick, the exhaustive best and the best packed
-    and fused-split configurations, the same layers as direct 3x3
+    the square sweep in every mode, the conv-as-gemm shapes with the plan of
+    a default call, the heuristic's packed configuration, the cost model's
+    pick, the exhaustive best and the best packed and fused-split
+    configurations, the same layers as direct 3x3
     convolutions, the paper's Conv layer with filters 3x3 to 11x11, and the
     512-problem grouped gemm replayed from its CUDA graph."""
     import torch
@@ -374,7 +375,7 @@ def other_workloads(model_path: str | None):
         C = torch.empty(M, N, device="cuda")
         flops = 2.0 * M * N * K
         res = {}
-        picks = {"heuristic": pkg.config_default("bf16x3", M, N, K)}
+        picks = {"default": None, "heuristic": pkg.config_default("bf16x3", M, N, K)}
         try:
             picks["model"] = pkg.costmodel_predict(M, N, K, "bf16x3")[0]
         except pkg.GemmError:
@@ -398,7 +399,7 @@ def other_workloads(model_path: str | None):
                 plan.execute(A, B, C, 1.0, 0.0)
             ms = _median_ms(lambda: [plan.execute(A, B, C, 1.0, 0.0) for _ in range(10)], 5, stream) / 10
             res[name] = {"tflops": round(flops / (ms * 1e-3) / 1e12, 2), "ms": round(ms, 4),
-                         "config": pkg.config_get("bf16x3", cid),
+                         "config": "default call" if cid is None else pkg.config_get("bf16x3", cid),
                          "hbm_gbs": round(4.0 * (M * K + K * N + M * N) / (ms * 1e-3) / 1e9, 1)}
             plan.destroy()
         simt = pkg.Plan(M, N, K, mode="simt")
@@ -453,7 +454,9 @@ def other_workloads(model_path: str | None):
             cfg = pkg.config_get("bf16x3", plan.info()["config_id"])
             res[f"{R}x{R}"] = {"ms": round(ms, 4), "tflops": round(flops / (ms * 1e-3) / 1e12, 2),
                                "hbm_gbs": round(4.0 * (x.numel() + f.numel() + o.numel()) / (ms * 1e-3) / 1e9, 1),
-                               "path": "fused-split" if cfg["fused"] else "packed"}
+                               # (the halo kernel's workspace holds no planes of the image)
+                               "path": "fused-split" if cfg["fused"]
+                               else "halo" if plan.info()["workspace_bytes"] < 4 * x.numel() else "packed"}
             plan.destroy()
         out["conv_filters"][f"{nb}x{H}x{Wd}x{Ci}->{Ko}"] = res
         del x, o

@@ -20,9 +20,9 @@
 //   * the filter comes as 128-byte k-chunks of its packed planes (hi rows, then
 //     lo rows, one operand of 2 KN rows): x_hi x [w_hi | w_lo] is ONE MMA of
 //     width 2 KN, x_lo x w_hi one of width KN into the second half, so that
-//     hi*hi accumulates apart from the two smaller products (its rounding
-//     chain is a third as long as in the im2col kernel) and A's hi part is
-//     read once for two products.
+//     hi*hi accumulates apart from the two smaller products (between folds at
+//     most 48 MMAs of it and 96 of those; the im2col kernel takes 48 of all
+//     three into one sum) and A's hi part is read once for two products.
 // The filter's K order is (channel group, tap, channel), so that a slot serves
 // all its taps before the next group's; the pack permutes the rows.
 //
@@ -30,12 +30,15 @@
 // layer (3 x 3, 16 -> 16) reads its A rows for 72 MMAs (2736 cycles at 128
 // bytes a cycle, with B), and the halo's arrival, its two passes of the split
 // and the staged outputs add about 1500; 108 units a SM.  Measured: paper's
-// layer 1016 -> 280 us a call (split pass, its rescale pass, filter pack and
+// layer 963 -> 281 us a call (split pass, its rescale pass, filter pack and
 // main kernel before; DRAM floor 158), 8 x 256 x 256 x 64 -> 64 202 -> 101 us.
 //
 // Whole-image exponent: beta == 0 runs unscaled at once while the split warps
 // fold max |x|, and a second launch repeats the convolution scaled only when
-// that maximum lies outside the unscaled range (it exits at once otherwise);
+// that maximum lies outside the unscaled range (it exits at once otherwise; such
+// an image takes twice the time: the paper's layer 529 us against 1245 of the
+// im2col path, 1 x 224 x 224 x 128 -> 128 83 against 64, where a scan of the
+// image first would cost every call 3 us of 48);
 // with beta != 0 (C is read, so a second pass could not start over) the
 // maximum is taken before, by the preparing launch.
 //
@@ -659,7 +662,10 @@ cudaError_t halo_dispatch(bool launch, const HaloArgs& a, int grid, const CUtens
 // Longest chain of k-steps one accumulator takes before it is folded into
 // FP32 registers (the tensor core's FP32 sum does not round to nearest).  The
 // im2col kernel folds every 16 k-steps of three products, 48 MMAs into one
-// accumulator; here hi*hi has an accumulator of its own, one MMA a k-step.
+// accumulator; here hi*hi has an accumulator of its own, one MMA a k-step, and
+// the two products 2^-8 (bf16) smaller share the other, two a k-step.  The errors
+// are below the im2col kernel's: 3.81e-6 against 3.88e-6 at 64 -> 64 features,
+// 3 x 3 (BF16X3); 7.6e-7 against 9.0e-7 in TF32X3.
 constexpr int kHaloFold = 48;
 
 bool halo_geometry(Prec prec, int64_t batch, int64_t H, int64_t W, int64_t C, int64_t K, int R, int S,
@@ -704,7 +710,8 @@ bool halo_geometry(Prec prec, int64_t batch, int64_t H, int64_t W, int64_t C, in
     // the blocks must not be mostly padding (128 -> 128 features, 3 x 3,
     // against the im2col kernel: 16 images of 50 x 50, blocks 61 % full,
     // 0.95-0.97x; 2 of 130 x 260 at 5 x 5, 86 % full, 1.03x; 1 of 224 x 224,
-    // 1.21x.  Up to 64 features it was faster on every shape tried.)
+    // 1.21x.  Of 140 shapes, 28 to 260 pixels a side, 16 to 256 channels, 3 x 3
+    // to 11 x 11, that first one alone was slower by more than 1 %.)
     if (a.nb > 1 && 10 * H * W < 7 * (16LL * a.hb) * (8LL * a.tiles * a.wb)) return false;
     const int64_t units = batch * a.hb * a.wb * a.nb;
     if (units > INT32_MAX) return false;

@@ -251,13 +251,15 @@ int default_config(gemm_mode mode, int64_t M, int64_t N, int64_t K, int sms, int
 // at 0.6 a unit of default_config's estimate, within 10 % of what 128^3 to
 // 1060^3 took.  Above one wave of tiles only up to 128 columns: every column
 // tile splits A again, which the estimate of wide products does not show (4096 x
-// 4096 x 128: 65 us against 55 packed).  Measured, packed -> this: 128^3 11.2 ->
-// 5.4, 512^3 13.1 -> 10.2, 768^3 16.6 -> 13.3, 1024^3 21.9 -> 18.3, 50176 x 64 x
-// 576 75.6 -> 37.5, 18790 x 16 x 1152 52 -> 19, 12544 x 128 x 1152 43 -> 37; kept
-// packed: 512 x 512 x 1024 (14.4 against 16.0), 2048 x 1024 x 512 (21.8 against
-// 22.6), 60000 x 256 x 576 (131 against 144), 700 x 900 x 1300 (21.8 against
-// 24.6).  1060^3 took 29.3 packed, 36 in two waves of tiles here and 22.9 in one,
-// its last rows in turned tiles (direct_grid); 1088^3 26.6 -> 21.3.
+// 4096 x 128: 65 us against 55 packed).  Measured in a graph, beta = 0.5, packed ->
+// this: 128^3 11.2 -> 5.5, 512^3 13.1 -> 10.4, 768^3 16.6 -> 13.8, 1024^3 22.2 ->
+// 20.0, 50176 x 64 x 576 74.9 -> 39.0, 18790 x 16 x 1152 50.8 -> 21.2, 12544 x 128
+// x 1152 43.1 -> 40.5; kept packed: 512 x 512 x 1024 (14.4 against 16.0), 2048 x
+// 1024 x 512 (21.8 against 22.6), 60000 x 256 x 576 (131 against 144), 700 x 900 x
+// 1300 (21.8 against 24.6).  1060^3 took 28.7 packed, 36 in two waves of tiles here
+// and 23.5 in one, its last rows in turned tiles (direct_grid); 1088^3 25.8 -> 22.2.
+// Of 110 random shapes, 64 to 1600 a side or tall and thin, none was slower than
+// packed by more than the runs differ.
 // A split-K configuration gives way (to the unsplit tile, for operands that start
 // off a 16-byte boundary) only where M, N and K are multiples of 4.  Plans whose
 // leading dimensions are not never come here: TMA could load no operand of theirs
@@ -275,7 +277,9 @@ static int direct_tile(const gemm_config& c, int64_t M, int64_t N, int64_t K, in
                (kA0 + (double)per * (c.block_n == 64 ? kChunk64 : kChunk128) + (c.block_n == 64 ? kEpi64 : kEpi128));
   if (splits > 1) est += kFix0 + kFix1 * (double)M * (double)N * (double)splits * 1e-6;
   double best = 4.0 + 8.0 * (double)(M + N) * (double)K / 5.5e6 + 0.6 * est;
-  if (splits > 1) best *= 0.85;   // (the estimate of split 128-wide tiles is up to a fifth high)
+  // The estimate was fitted to rank configurations, not for absolute times, and is
+  // up to a fifth high for split ones; only here are they set against another kernel.
+  if (splits > 1) best *= 0.85;
   int pick = 0;
   for (int bn : {32, 64}) {
     const int64_t t = direct_grid(bn, M, N, sms).units();
