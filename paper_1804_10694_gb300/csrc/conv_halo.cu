@@ -21,7 +21,7 @@
 //     lo rows, one operand of 2 KN rows): x_hi x [w_hi | w_lo] is ONE MMA of
 //     width 2 KN, x_lo x w_hi one of width KN into the second half, so that
 //     hi*hi accumulates apart from the two smaller products (between folds at
-//     most 48 MMAs of it and 96 of those; the im2col kernel takes 48 of all
+//     most 44 MMAs of it and 88 of those; the im2col kernel takes 48 of all
 //     three into one sum) and A's hi part is read once for two products.
 // The filter's K order is (channel group, tap, channel), so that a slot serves
 // all its taps before the next group's; the pack permutes the rows.
@@ -663,10 +663,13 @@ cudaError_t halo_dispatch(bool launch, const HaloArgs& a, int grid, const CUtens
 // FP32 registers (the tensor core's FP32 sum does not round to nearest).  The
 // im2col kernel folds every 16 k-steps of three products, 48 MMAs into one
 // accumulator; here hi*hi has an accumulator of its own, one MMA a k-step, and
-// the two products 2^-8 (bf16) smaller share the other, two a k-step.  The errors
-// are below the im2col kernel's: 3.81e-6 against 3.88e-6 at 64 -> 64 features,
-// 3 x 3 (BF16X3); 7.6e-7 against 9.0e-7 in TF32X3.
-constexpr int kHaloFold = 48;
+// the two small products share the other, two a k-step.  With 48 k-steps a fold
+// the TF32X3 errors were a little above the im2col kernel's (128 -> 64 features,
+// 3 x 3, 144 k-steps: 9.27e-7 against 9.10e-7); with 44 they are below it on every
+// shape tried (7.04e-7 there, 8.4e-7 against 9.0e-7 at 64 -> 64, 7 x 7), in BF16X3
+// 3.80e-6 against 3.85e-6.  The one more fold costs 0.3 to 0.9 % there and nothing
+// elsewhere; 40 would cost 1 % at 9 x 9.
+constexpr int kHaloFold = 44;
 
 bool halo_geometry(Prec prec, int64_t batch, int64_t H, int64_t W, int64_t C, int64_t K, int R, int S,
                    HaloArgs* out) {

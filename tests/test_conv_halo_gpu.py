@@ -125,3 +125,26 @@ def test_ragged_columns_many_units(mode, shape, beta):
         assert np.array_equal(do.cpu().numpy(), want)
     plan.destroy()
     pkg.device_error()
+
+
+@pytest.mark.parametrize("mode", ["bf16x3", "tf32x3"])
+@pytest.mark.parametrize("shape", [(8, 112, 112, 128, 64, 3, 3), (8, 112, 112, 64, 64, 7, 7), (8, 112, 112, 16, 16, 3, 3)])
+def test_as_accurate_as_the_im2col_kernel(mode, shape):
+    """Folds are short enough that the error against 64 bits is no larger than
+    that of the im2col kernel on the same layer (its configuration named)."""
+    n, H, Wd, C, K, R, S = shape
+    g = torch.Generator(device="cuda").manual_seed(340)
+    x, f = (torch.empty(s, device="cuda").uniform_(-1, 1, generator=g) for s in ((n, H, Wd, C), (R, S, C, K)))
+    pad = torch.nn.functional.pad(x.double(), (0, 0, S // 2, S // 2, R // 2, R // 2))
+    exact = torch.zeros(n * H * Wd, K, dtype=torch.float64, device="cuda")
+    for r in range(R):
+        for s in range(S):
+            exact.addmm_(pad[:, r:r + H, s:s + Wd].reshape(-1, C), f[r, s].double())
+    err = []
+    for named in (False, True):
+        plan = pkg.ConvPlan(n, H, Wd, C, K, R, S, mode=mode, config_id=config if named else None)
+        config = plan.info()["config_id"]
+        out = plan.execute(x, f, torch.empty(n, H, Wd, K, device="cuda"))
+        err.append((out.view(-1, K).double() - exact).norm().item())
+        plan.destroy()
+    assert err[0] <= err[1]
