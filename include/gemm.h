@@ -232,8 +232,10 @@ gemm_status gemm_plan_create_t(int transA, int transB, int64_t M, int64_t N, int
  * config_id < 0 picks the default: packed where it applies (C a multiple of
  * 16; BF16X6 has no fused-split kernel), else fused-split.  A default packed
  * BF16X3 or TF32X3 plan without split-K and with at least nine taps runs the
- * halo kernel where its tiles fit: the image is read once as FP32 and split
- * in shared memory, its workspace holds the filter's planes only; the other
+ * halo kernel where its tiles fit and an estimate finds it faster (not for
+ * images that are mostly the padding of its 16 x 16 or 16 x 32 blocks): the
+ * image is read once as FP32 and split in shared memory, its workspace holds
+ * the filter's planes only; the other
  * default packed plans with at most 32 output features (K <= 32) and no
  * split-K run 128 x 32 tiles, two CTAs a SM where shared memory holds two.
  * One power-of-two exponent covers the whole image (its max |x|); B is scaled

@@ -671,6 +671,37 @@ cudaError_t halo_dispatch(bool launch, const HaloArgs& a, int grid, const CUtens
 // elsewhere; 40 would cost 1 % at 9 x 9.
 constexpr int kHaloFold = 44;
 
+// Whether the halo kernel is the faster one: its estimate against that of the im2col
+// kernel with tiles of 128 x bn, ctas of them at a time on a SM.  Both in
+// microseconds: a constant, and waves of units (tiles) at what a group of 16 channels
+// of one takes: here the split of its halo's pixels and its MMAs (taps x tiles), there
+// loads and MMAs of its taps.  Fitted to 1152 shapes (9 to 500 pixels a side, 1 to 200
+// images, 16 to 128 channels and 16 to 192 features, 3 x 3 to 11 x 11, both betas; rms
+// 4 to 8 %).  Blocks that are mostly padding, or a last wave that the im2col tiles do
+// not need, make it the slower one.  The im2col kernel then folds twice as often as by
+// default, for errors no larger than this one's, which costs it up to 8 %: hence the
+// margin.  64 images of 17 x 17 x 64 -> 64, 11 x 11: 140 -> 89 us; 16 of 56 x 56 x 128 ->
+// 128, 3 x 3 in TF32X3: 122 -> 106; the 58 shapes sent away 1.20 times as fast on average,
+// none slower.
+bool halo_pays(Prec prec, const HaloArgs& a, int64_t batch, int bn, int ctas, int sms) {
+  struct Cost {
+    double fixed, tap;   // halo: per 1000 pixels, per tap and tile; im2col: per group, per tap
+  };
+  static constexpr Cost kHalo[2][3] = {{{0.60, 0.046}, {0.96, 0.050}, {1.04, 0.060}},     // 16, 32, 64 features a unit
+                                       {{1.39, 0.100}, {3.42, 0.096}, {4.59, 0.109}}};
+  static constexpr Cost kIm2col[2][3] = {{{0.22, 0.219}, {0.17, 0.140}, {0.64, 0.150}},   // tiles 32, 64, 128 wide
+                                         {{0.73, 0.377}, {0.42, 0.307}, {0.93, 0.313}}};
+  const int tf32 = prec == Prec::TF32, taps = a.R * a.S;
+  const Cost h = kHalo[tf32][a.kn == 16 ? 0 : a.kn == 32 ? 1 : 2], i = kIm2col[tf32][bn == 32 ? 0 : bn == 64 ? 1 : 2];
+  const int64_t slots = static_cast<int64_t>(sms) * ctas;
+  const int64_t tiles = ((batch * a.H * a.W + 127) / 128) * ((a.K + bn - 1) / bn);
+  const double hwaves = static_cast<double>((a.units + sms - 1) / sms);
+  const double iwaves = static_cast<double>((tiles + slots - 1) / slots);
+  const double halo = 16.0 + hwaves * a.groups * (h.fixed * a.px / 1000.0 + h.tap * taps * a.tiles);
+  const double im2col = 22.0 + (iwaves - 0.2) * a.groups * (i.fixed + i.tap * taps);
+  return halo <= (tf32 ? 1.08 : 1.11) * im2col;
+}
+
 bool halo_geometry(Prec prec, int64_t batch, int64_t H, int64_t W, int64_t C, int64_t K, int R, int S,
                    HaloArgs* out) {
   // (a filter chunk of four k-steps meets at most one group's end with nine taps or more)

@@ -134,6 +134,9 @@ struct HaloArgs {
 // Whether the kernel covers this convolution; fills the geometry.
 bool halo_geometry(Prec prec, int64_t batch, int64_t H, int64_t W, int64_t C, int64_t K, int R, int S,
                    HaloArgs* out);
+// Whether it is the faster one for that geometry, against the im2col kernel with
+// tiles of 128 x bn, `ctas` a SM.
+bool halo_pays(Prec prec, const HaloArgs& a, int64_t batch, int bn, int ctas, int sms);
 // Raise the kernel variant's shared-memory limit (call outside stream capture).
 cudaError_t halo_prepare(Prec prec, const HaloArgs& a);
 // tmX: FP32 image {C, W, H, N}, boxes of 16 channels x bw x (16 + R - 1);

@@ -1437,8 +1437,14 @@ gemm_status gemm_conv_plan_create(int64_t batch, int64_t H, int64_t W, int64_t C
   // features and no split-K takes the narrow tile (128 x 32, two CTAs a SM)
   const unsigned narrow = default_choice && packed_conv && K <= 32 && c.split_k == 1 ? kOptNarrowConv : 0u;
   HaloArgs geo{};
-  const bool halo = default_choice && packed_conv && c.split_k == 1 &&
-                    halo_geometry(prec_of_mode(mode), batch, H, W, C, K, R, S, &geo);
+  bool halo = default_choice && packed_conv && c.split_k == 1 &&
+              halo_geometry(prec_of_mode(mode), batch, H, W, C, K, R, S, &geo);
+  if (halo && !halo_pays(prec_of_mode(mode), geo, batch, narrow ? 32 : c.block_n,
+                         narrow ? tc_narrow_ctas_per_sm(prec_of_mode(mode)) : 1, dev->sms)) {
+    halo = false;
+    config_id = find_config(c.block_n, 1, 2, c.group_m);   // folds every two chunks: as accurate
+    config_get(mode, config_id, &c);
+  }
   gemm_plan_t p = nullptr;
   gemm_status st = plan_create_impl(M, K, Kd, Kd, K, K, mode, config_id, GEMM_SELECT_DEFAULT, &p, false,
                                     false, packed_conv ? elems : -1, narrow, halo ? &geo : nullptr);

@@ -148,3 +148,28 @@ def test_as_accurate_as_the_im2col_kernel(mode, shape):
         err.append((out.view(-1, K).double() - exact).norm().item())
         plan.destroy()
     assert err[0] <= err[1]
+
+
+@pytest.mark.parametrize("mode,shape", [("bf16x3", (64, 17, 17, 64, 64, 11, 11)), ("tf32x3", (64, 17, 17, 64, 64, 3, 3)),
+                                        ("tf32x3", (64, 17, 17, 128, 48, 5, 5)), ("tf32x3", (64, 28, 28, 128, 128, 3, 3))])
+def test_mostly_padding_runs_the_im2col_kernel(mode, shape):
+    """Images that fill little of the halo kernel's blocks, or need a wave more
+    of them, keep the im2col kernel, with folds short enough for errors no
+    larger than those of its own default."""
+    n, H, Wd, C, K, R, S = shape
+    x = W.conv_image(n, H, Wd, C, 350)
+    f = W.conv_filter(C, K, 351, R=R, S=S)
+    ref = conv.conv_f64(x, f)
+    dx, df = torch.from_numpy(x).cuda(), torch.from_numpy(f).cuda()
+    plan = pkg.ConvPlan(n, H, Wd, C, K, R, S, mode=mode)
+    info = plan.info()
+    assert info["workspace_bytes"] > (4 if mode == "bf16x3" else 8) * x.size   # the image's planes
+    cfg = pkg.config_get(mode, info["config_id"])
+    usual = next(i for i in range(pkg.config_count(mode)) if pkg.config_get(mode, i) == {**cfg, "kb": 4})
+    err = []
+    for p in (plan, pkg.ConvPlan(n, H, Wd, C, K, R, S, mode=mode, config_id=usual)):
+        out = p.execute(dx, df, torch.empty(n, H, Wd, K, device="cuda")).cpu().numpy()
+        err.append(oracle.rel_frob(out.reshape(-1, K), ref.reshape(-1, K)))
+        p.destroy()
+    assert err[0] <= err[1] <= TOL
+    pkg.device_error()
