@@ -24,7 +24,8 @@
 // 128 rows of A and BN columns of B; if either lies outside the unscaled range
 // the tile is computed once more with the exponents (nothing has been stored
 // by then), its values read straight from global memory, so that the ring's
-// loads for the next tile stay where they are.
+// loads for the next tile stay where they are.  (1024^3 with all of A out of the
+// range takes 53 us for 19, packed 53; with one block of 128 rows 53, packed 42.)
 //
 // Bounded by shared-memory bandwidth (an item of a 128 x 64 tile crosses it four
 // times: copied in, read, written as parts, read by the MMAs, about 850 cycles;
