@@ -58,7 +58,7 @@ def test_host_calls_use_the_shape_s_own_plan():
     free = torch.cuda.mem_get_info()[0]
     for beta in (0.5, 0.0, 0.5):
         pkg.gemm_host(A, B, C.clone().pin_memory(), 1.5, beta, mode="bf16x3", stream=s)
-    assert torch.cuda.mem_get_info()[0] == free
+    assert torch.cuda.mem_get_info()[0] >= free
     with torch.cuda.graph(graph, stream=s):
         pkg.gemm(a, b, c, 1.5, 0.5, mode="bf16x3", stream=s)
     graph.replay()
