@@ -483,8 +483,9 @@ __global__ void __launch_bounds__(kDirThreads, 1)
             // its reads before the next copy into it (another proxy's writes; an
             // arrival right behind the reads let the copy overtake some of them).
             // The fence costs 2 to 3 %.  Given back behind the parts' fence alone,
-            // the stage is late for tall products: 50176 x 64 x 576 40.7 us against
-            // 35.7 (512^3 9.8 against 10.4).
+            // the stage is late for operands that come from HBM: 50176 x 64 x 576
+            // 40.7 us against 35.7, 512^3 on cold inputs 16.4 against 14.4 (9.8
+            // against 10.4 where L2 holds them).
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(sempty(sg));
